@@ -96,8 +96,14 @@ bool mt::valid_poly(int kind, int l, int n) {
   return false;
 }
 
+bool mt::fixed_point_poly(int kind, int l, int n) {
+  const bool pm_i = n % 2 == 0 && ((kind == 1 && l == 2) || (kind == 2 && l >= 2));
+  return !pm_i;
+}
+
 PolyDev mt::make_poly(int kind, int l, int n) {
   PolyDev P;
+  P.fx = fixed_point_poly(kind, l, n) ? 1 : 0;
   P.kind = kind;
   P.l = l;
   P.n = n;
@@ -235,10 +241,21 @@ bool make_plan(int kind, int l, int n, const mt_options* o, int retry, Plan* pl)
     N0 = std::min<int64_t>(int64_t(1) << 17,
                            std::max<int64_t>(Md / 128, std::min<int64_t>(int64_t(1) << 15, Md / 16)));
     N0 = std::max<int64_t>(N0, std::min<int64_t>(int64_t(1) << 18, Md >> 12));
-  } else {
-    // binary64: the walk already keeps the binary64 pipe busy; more chunks
-    // would only add seed lifts
+  } else if (!p.P.fx) {
+    // in binary64 arithmetic: the walk already keeps that pipe busy; more
+    // chunks would only add seed lifts
     N0 = std::min<int64_t>(int64_t(1) << 15, Md / 16);
+  } else {
+    // binary64 in fixed point: the walk is latency-bound with one lane per chunk
+    // until some 2^15 lanes fill the integer pipes, and a seed costs about as
+    // much as 8 sqrt(Md) / 2^8 sub-steps' share of it.  Chunks of 8 sub-steps
+    // up to 2^14 lanes, then as many lanes as sqrt(Md) 2^4 (measured, ms a
+    // split: p_12 0.455 -> 0.42, p_16 0.62 -> 0.58, p_20 2.37 -> 2.17, p_22 8.1
+    // -> 7.0, p_24 32.8 -> 26.2 against 2^14 lanes at most)
+    N0 = std::min<int64_t>(int64_t(1) << 15, Md / 8);
+    int lg = 0;
+    while ((int64_t(1) << lg) < Md) ++lg;
+    N0 = std::max<int64_t>(N0, std::min<int64_t>(Md / 8, int64_t(1) << std::min(18, 5 + lg / 2)));
   }
   // streamed split: when the upper half holds more than 2^31 starts (the
   // root-set indices are 32-bit), or when asked for

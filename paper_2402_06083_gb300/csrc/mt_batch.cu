@@ -11,6 +11,7 @@
 // (k_descend's scheme, each lane looking up the polynomial of the start it
 // pops), then one sort by (polynomial, Re) and the segmented root-set,
 // type and certificate kernels (SegView).
+#include "mt_descent.cuh"
 #include "mt_levelline.cuh"
 
 namespace mt {
@@ -40,25 +41,26 @@ __global__ void k_seed_lift_batch(const BatchEntry* __restrict__ E, const int64_
 }
 
 // persistent: lanes pop level-line chunks of any polynomial from one queue
+template <int FB>
 __global__ void k_walk_batch(const BatchEntry* __restrict__ E, const int64_t* __restrict__ chunk_off,
                              int np, int64_t total, double lambda0, int M, int every,
                              const double2* __restrict__ seeds, double2* __restrict__ starts,
                              DevCounters* ctr) {
   __shared__ double2 ph[64];
-  for (int q = threadIdx.x; q < M; q += blockDim.x) {
-    double c, s;
-    unit_phase((uint64_t)q, (uint64_t)M, c, s);
-    ph[q] = make_double2(lambda0 * c, lambda0 * s);
-  }
-  __syncthreads();
+  __shared__ longlong2 phx[64];
+  walk_phases<FB>(lambda0, M, ph, phx);
   unsigned long long steps = 0, fails = 0;
   for (;;) {
     const int64_t c = (int64_t)atomicAdd(&ctr->queue_head2, 1ull);
     if (c >= total) break;
     const int p = find_seg(chunk_off, np, c);
     const BatchEntry e = E[p];
-    fails += walk_chunk(e.P, ph, M, every, e.L, e.nchunks, c - chunk_off[p], seeds + e.seed_off,
-                        starts + e.start_off, steps) ? 1 : 0;
+    const int64_t j = c - chunk_off[p];
+    const double2* sd = seeds + e.seed_off;
+    fails += walk_chunk_from<FB, true>(e.P, lambda0, M, every, e.L, e.nchunks, j, sd[j], sd[j + 1], ph, phx,
+                                       starts + e.start_off, steps)
+                 ? 1
+                 : 0;
   }
   warp_add_u64(&ctr->walk_newton, steps);
   warp_add_u64(&ctr->walk_fail, fails);
@@ -68,7 +70,7 @@ __global__ void k_walk_batch(const BatchEntry* __restrict__ E, const int64_t* __
 // with the polynomial looked up per start)
 __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restrict__ E,
                                                        const int64_t* __restrict__ start_off,
-                                                       int np, int64_t count, double tol2,
+                                                       int np, int64_t count, float tol2,
                                                        const double2* __restrict__ starts,
                                                        double2* __restrict__ cand,
                                                        uint8_t* __restrict__ status,
@@ -76,61 +78,55 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
                                                        DevCounters* ctr) {
   const unsigned lane = threadIdx.x & 31;
   int64_t idx = -1;
-  double zr = 0.0, zi = 0.0, rdiv2 = 16.0, prev2 = 1e300;
-  int it = 0, m = 1, lcap = -1, cap = 20;
+  Descent d{0, 0, 16.f, 3.0e38f, 0, false, true};
+  int m = 1, lcap = -1, cap = 20, outcome = -1;
   unsigned long long steps = 0, orbit = 0, nconv = 0, ndiv = 0, nto = 0;
+  bool drained = false;
   for (;;) {
-    const unsigned need = __ballot_sync(0xffffffffu, idx < 0);
-    if (need) {
-      unsigned long long base = 0;
-      if (lane == (unsigned)(__ffs(need) - 1))
-        base = atomicAdd(&ctr->queue_head, (unsigned long long)__popc(need));
-      base = __shfl_sync(0xffffffffu, base, __ffs(need) - 1);
-      if (idx < 0) {
-        idx = (int64_t)(base + __popc(need & lanemask_lt()));
-        if (idx < count) {
-          const int p = find_seg(start_off, np, idx);
-          const BatchEntry e = E[p];
-          m = e.P.m;
-          lcap = e.P.lcap;
-          cap = e.cap;
-          seg[idx] = (uint16_t)p;
-          const double2 z0 = starts[idx];
-          zr = z0.x;
-          zi = z0.y;
-          it = 0;
-          prev2 = 1e300;
-          rdiv2 = fmax(16.0, 4.0 * fma(zr, zr, zi * zi));
-        }
-      }
-    }
-    const bool active = idx >= 0 && idx < count;
-    if (!__any_sync(0xffffffffu, active)) break;
-    if (active) {
-      double vr, vi, dr, di;
-      orbit_f64(m, lcap, 1.0, zr, zi, vr, vi, dr, di);
-      double qr, qi;
-      cdiv_f64(vr, vi, dr, di, qr, qi);
-      zr -= qr;
-      zi -= qi;
-      ++it;
-      ++steps;
-      orbit += (unsigned)m;
-      const double s2 = fma(qr, qr, qi * qi);
-      int outcome = -1;
-      if (!finite2(zr, zi) || fma(zr, zr, zi * zi) > rdiv2) outcome = 1;
-      else if (s2 < tol2) outcome = 0;
-      else if (s2 >= 0.25 * prev2 && s2 < floor2_f64(zr, zi)) outcome = 0;
-      else if (it >= cap) outcome = 2;
-      prev2 = s2;
+    // as k_descend: written and refilled together once DESC_REFILL lanes wait
+    const unsigned running = __ballot_sync(0xffffffffu, idx >= 0 && idx < count && outcome < 0);
+    const unsigned wait = __popc(__ballot_sync(0xffffffffu, idx < 0 || outcome >= 0));
+    if (wait >= DESC_REFILL || running == 0u) {
       if (outcome >= 0) {
-        cand[idx] = make_double2(zr, zi);
+        cand[idx] = descent_point(d);
         status[idx] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
         nto += outcome == 2;
+        outcome = -1;
         idx = -1;
       }
+      const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
+      if (need) {
+        unsigned long long base = 0;
+        if (lane == (unsigned)(__ffs(need) - 1))
+          base = atomicAdd(&ctr->queue_head, (unsigned long long)__popc(need));
+        base = __shfl_sync(0xffffffffu, base, __ffs(need) - 1);
+        drained = (int64_t)(base + __popc(need)) >= count;
+        if (idx < 0) {
+          idx = (int64_t)(base + __popc(need & lanemask_lt()));
+          if (idx < count) {
+            const int p = find_seg(start_off, np, idx);
+            const BatchEntry e = E[p];
+            m = e.P.m;
+            lcap = e.P.lcap;
+            cap = e.cap;
+            seg[idx] = (uint16_t)p;
+            descent_start(d, starts[idx], e.P.fx != 0);
+          }
+        }
+      }
+      if (drained && idx < 0) idx = count;
+    }
+    const bool active = idx >= 0 && idx < count && outcome < 0;
+    if (!__any_sync(0xffffffffu, active)) {
+      if (drained && !__any_sync(0xffffffffu, outcome >= 0)) break;
+      continue;
+    }
+    if (active) {
+      outcome = descent_step<true>(m, lcap, d, tol2, cap);
+      ++steps;
+      orbit += (unsigned)m;
     }
   }
   warp_add_u64(&ctr->desc_newton, steps);
@@ -168,13 +164,15 @@ cudaError_t launch_walk_batch(const BatchEntry* E, const int64_t* chunk_off, int
   if (total <= 0) return cudaSuccess;
   const int bs = 64;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_walk_batch, bs, 0);
+  const int fb = lambda0 <= 12.0 ? 28 : lambda0 <= 200.0 ? 26 : 0;  // as walk_fb
+  const auto kern = fb == 28 ? &k_walk_batch<28> : fb == 26 ? &k_walk_batch<26> : &k_walk_batch<0>;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, bs, 0);
   if (e != cudaSuccess) return e;
   int64_t grid = (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
   const int64_t need = (total + bs - 1) / bs;
   if (grid > need) grid = need;
   MT_COUNT_LAUNCH(1);
-  k_walk_batch<<<(unsigned)grid, bs, 0, s>>>(E, chunk_off, np, total, lambda0, M, every, seeds, starts,
+  kern<<<(unsigned)grid, bs, 0, s>>>(E, chunk_off, np, total, lambda0, M, every, seeds, starts,
                                              ctr);
   return cudaGetLastError();
 }
@@ -187,12 +185,11 @@ cudaError_t launch_descend_batch(const BatchEntry* E, const int64_t* start_off, 
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_descend_batch, bs, 0);
   if (e != cudaSuccess) return e;
-  if (per_sm > 2) per_sm = 2;  // 8 warps/SM saturate the binary64 pipe (as launch_descend)
   int64_t grid = (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
   const int64_t need = (count + bs - 1) / bs;
   if (grid > need) grid = need;
   MT_COUNT_LAUNCH(1);
-  k_descend_batch<<<(unsigned)grid, bs, 0, s>>>(E, start_off, np, count, tol * tol, starts, cand,
+  k_descend_batch<<<(unsigned)grid, bs, 0, s>>>(E, start_off, np, count, tol2_f(tol), starts, cand,
                                                 status, seg, ctr);
   return cudaGetLastError();
 }

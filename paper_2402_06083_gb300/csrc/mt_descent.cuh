@@ -1,0 +1,115 @@
+// mt_descent.cuh -- one binary64 Newton descent in fixed point (mt_fix.cuh),
+// shared by the single-polynomial kernels (mt_newton.cu) and the batched
+// one (mt_batch.cu).
+#pragma once
+#include "mt_common.cuh"
+#include "mt_fix.cuh"
+
+namespace mt {
+
+constexpr int FXB = 28;  // fraction bits of the high limb: |Re|, |Im| < 4
+// waiting lanes that trigger a refill of the persistent kernels (p_24: 1 13.66
+// ms, 3 13.54, 5 13.60, 8 13.99; every s_{l,n} to order 16: 1.13, 1.09, 1.09, 1.10)
+constexpr unsigned DESC_REFILL = 3;
+
+// z as X, Y at 2^-60, or as the bits of its binary64 coordinates (wide:
+// outside the fixed range, or a polynomial kept in binary64), and the squares of the last step and of the
+// divergence radius.
+struct Descent {
+  long long X, Y;
+  float rdiv2, prev2;
+  int it;
+  bool wide, fx;
+};
+
+__device__ __forceinline__ void descent_set(Descent& d, double x, double y) {
+  d.wide = !(d.fx && fx_fits<FXB>(x) && fx_fits<FXB>(y));
+  d.X = d.wide ? __double_as_longlong(x) : fx_from_f64<FXB>(x);
+  d.Y = d.wide ? __double_as_longlong(y) : fx_from_f64<FXB>(y);
+}
+__device__ __forceinline__ void descent_start(Descent& d, double2 z0, bool fx) {
+  d.fx = fx;
+  d.it = 0;
+  d.prev2 = 3.0e38f;
+  // long jump: beyond twice the start radius and outside D(0, 4)
+  const float ax = f32_trunc(z0.x), ay = f32_trunc(z0.y);
+  d.rdiv2 = fmaxf(16.f, 4.f * fmaf(ax, ax, ay * ay));
+  descent_set(d, z0.x, z0.y);
+}
+__device__ __forceinline__ double2 descent_point(const Descent& d) {
+  return d.wide ? make_double2(__longlong_as_double(d.X), __longlong_as_double(d.Y))
+                : make_double2(fx_to_f64<FXB>(d.X), fx_to_f64<FXB>(d.Y));
+}
+
+// One binary64 Newton step, for the points outside the fixed range (starts of
+// polynomials of a small degree), at a zero of P', or of a polynomial kept in
+// binary64; NaN where it is not
+// finite.  s2 receives |step|^2.
+static __device__ __noinline__ double2 newton_step_f64(int m, int lcap, double2 z, float& s2) {
+  double vr, vi, dr, di, qr, qi;
+  orbit_f64(m, lcap, 1.0, z.x, z.y, vr, vi, dr, di);
+  cdiv_f64(vr, vi, dr, di, qr, qi);
+  const float fr = f32_trunc(qr), fi = f32_trunc(qi);
+  s2 = fmaf(fr, fr, fi * fi);
+  return make_double2(z.x - qr, z.y - qi);
+}
+
+// One Newton step and its outcome: -1 go on, 0 converged, 1 divergent, 2 cap.
+template <bool CAP>
+__device__ __forceinline__ int descent_step(int m, int lcap, Descent& d, float tol2, int cap) {
+  float s2 = 0.f;
+  bool ok = false;
+  if (!d.wide) {
+    FxVal o;
+    const FxTarget T{0, 0, ff{0.f, 0.f}, ff{0.f, 0.f}, true};
+    fx_eval<FXB, CAP>(m, lcap, 8, d.X, d.Y, T, o);
+    ff qr, qi;
+    fx_cmul(o.nr, o.ni, o.ir, o.ii, o.sc, qr, qi);
+    ok = fabsf(qr.hi) < 4.f && fabsf(qi.hi) < 4.f;  // false for NaN too
+    if (o.over) {  // P or P' beyond binary64
+      d.X = d.Y = 0x7ff8000000000000ll;
+      d.wide = true;
+      ok = true;
+    } else if (ok) {
+      s2 = fmaf(qr.hi, qr.hi, qi.hi * qi.hi);
+      d.X -= fx_from_ff<FXB>(qr);
+      d.Y -= fx_from_ff<FXB>(qi);
+      if (!(fx_in<FXB>(d.X) && fx_in<FXB>(d.Y))) {
+        d.X = __double_as_longlong(fx_to_f64<FXB>(d.X));
+        d.Y = __double_as_longlong(fx_to_f64<FXB>(d.Y));
+        d.wide = true;
+      }
+    }
+  }
+  if (!ok) {
+    const double2 z = newton_step_f64(m, lcap, descent_point(d), s2);
+    descent_set(d, z.x, z.y);
+  }
+  float ax, ay;
+  if (d.wide) {  // inf or NaN stays so
+    ax = f32_trunc(__longlong_as_double(d.X));
+    ay = f32_trunc(__longlong_as_double(d.Y));
+  } else {
+    ax = (float)fx_hi(d.X) * (1.f / (1 << FXB));
+    ay = (float)fx_hi(d.Y) * (1.f / (1 << FXB));
+  }
+  ++d.it;
+  int outcome = -1;
+  const float fl = (1.f + fabsf(ax) + fabsf(ay)) * 3.552713678800501e-15f;  // 16 ulp of binary64
+  const float z2 = fmaf(ax, ax, ay * ay);
+  if (!(z2 <= d.rdiv2) || z2 > 3.0e38f) outcome = 1;
+  else if (s2 < tol2) outcome = 0;  // the step that met tol also squared the error
+  // binary64 rounding floor: steps stopped shrinking within a few ulp of z
+  // (between two close roots Newton also stalls, at |step| ~ their
+  // separation^2 / distance, far above this floor)
+  else if (s2 >= 0.25f * d.prev2 && s2 < fl * fl) outcome = 0;
+  else if (d.it >= cap) outcome = 2;
+  d.prev2 = s2;
+  return outcome;
+}
+
+// tol^2 in binary32 (not below its smallest positive value, so that a step
+// of zero always meets it)
+inline float tol2_f(double tol) { return std::max((float)(tol * tol), 1.4e-45f); }
+
+}  // namespace mt

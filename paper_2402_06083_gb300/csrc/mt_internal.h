@@ -16,6 +16,7 @@ struct PolyDev {
   int m;
   int lcap;
   int log2d;  // deg P = 2^log2d
+  int fx;     // 1: the binary64 tier runs in fixed point (fixed_point_poly)
 };
 
 // Device-side counters of one split (zeroed at the start of a call).
@@ -76,6 +77,12 @@ struct BatchEntry {
 // The polynomial domain (kind 0: p_n, 1: s_{l,n}, 2: q_{l,n}) and the
 // kernel descriptor of a polynomial in it.
 bool valid_poly(int kind, int l, int n);
+// Whether the binary64 tier's orbits of a polynomial run in fixed point
+// (mt_fix.cuh): all but those with the roots 0 and +-i -- s_{2,n} and q_{l,n},
+// l >= 2, with n even, where +-i are the points of type (2, 2) -- whose equal
+// real parts leave their order in the (Re, Im) list to the last digits of
+// the binary64 descents.
+bool fixed_point_poly(int kind, int l, int n);
 PolyDev make_poly(int kind, int l, int n);
 
 // Per-kernel timing: CUDA events recorded around single launches on the

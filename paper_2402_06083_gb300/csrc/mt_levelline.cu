@@ -30,41 +30,21 @@ __global__ void k_seed_lift(PolyDev P, double lambda0, int64_t N0, int log2N0, i
   warp_add_u64(&ctr->seed_newton, steps);
 }
 
-__global__ void k_walk(PolyDev P, double lambda0, int M, int every, int64_t L, int64_t nchunks,
-                       const double2* __restrict__ seeds, double2* __restrict__ starts,
+// Chunks [j0, j0 + nch), starts written from index j0 L / every on (a
+// streamed split walks the level line a range of chunks at a time).
+template <int FB, bool CAP>
+__global__ void k_walk(PolyDev P, double lambda0, int M, int every, int64_t L, int64_t nchunks, int64_t j0,
+                       int64_t nch, const double2* __restrict__ seeds, double2* __restrict__ starts,
                        DevCounters* ctr) {
   __shared__ double2 ph[64];
-  for (int q = threadIdx.x; q < M; q += blockDim.x) {
-    double c, s;
-    unit_phase((uint64_t)q, (uint64_t)M, c, s);
-    ph[q] = make_double2(lambda0 * c, lambda0 * s);
-  }
-  __syncthreads();
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long steps = 0, fails = 0;
-  if (j < nchunks) fails = walk_chunk(P, ph, M, every, L, nchunks, j, seeds, starts, steps) ? 1 : 0;
-  warp_add_u64(&ctr->walk_newton, steps);
-  warp_add_u64(&ctr->walk_fail, fails);
-}
-
-// Chunks [j0, j0 + nch) only, starts written from index j0 L / every on
-// (streamed splits, which walk the level line a range of chunks at a time).
-__global__ void k_walk_range(PolyDev P, double lambda0, int M, int every, int64_t L, int64_t nchunks,
-                             int64_t j0, int64_t nch, const double2* __restrict__ seeds,
-                             double2* __restrict__ starts, DevCounters* ctr) {
-  __shared__ double2 ph[64];
-  for (int q = threadIdx.x; q < M; q += blockDim.x) {
-    double c, s;
-    unit_phase((uint64_t)q, (uint64_t)M, c, s);
-    ph[q] = make_double2(lambda0 * c, lambda0 * s);
-  }
-  __syncthreads();
+  __shared__ longlong2 phx[64];
+  walk_phases<FB>(lambda0, M, ph, phx);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long steps = 0, fails = 0;
   if (i < nch) {
     const int64_t j = j0 + i;
-    fails = walk_chunk_from(P, ph, M, every, L, nchunks, j, seeds[j], seeds[j + 1], starts, steps,
-                            j0 * L / every)
+    fails = walk_chunk_from<FB, CAP>(P, lambda0, M, every, L, nchunks, j, seeds[j], seeds[j + 1], ph, phx, starts,
+                                     steps, j0 * L / every)
                 ? 1
                 : 0;
   }
@@ -77,10 +57,17 @@ cudaError_t launch_walk_range(const PolyDev& P, double lambda0, int M, int every
                               cudaStream_t s, int block) {
   if (nch <= 0) return cudaSuccess;
   const int bs = (block >= 32 && block <= 1024 && block % 32 == 0) ? block : 64;
+  const int fb = walk_fb(P, lambda0);
+  const bool cap = P.lcap >= 1;
+  const auto kern = fb == 28 ? (cap ? &k_walk<28, true> : &k_walk<28, false>)
+                    : fb == 26 ? (cap ? &k_walk<26, true> : &k_walk<26, false>)
+                               : (cap ? &k_walk<0, true> : &k_walk<0, false>);
   MT_COUNT_LAUNCH(1);
-  k_walk_range<<<(unsigned)((nch + bs - 1) / bs), bs, 0, s>>>(P, lambda0, M, every, L, nchunks, j0, nch, seeds,
-                                                              starts, ctr);
-  return cudaGetLastError();
+  cudaError_t e = ktimer_begin(KS_WALK, s);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)((nch + bs - 1) / bs), bs, 0, s>>>(P, lambda0, M, every, L, nchunks, j0, nch, seeds, starts, ctr);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return ktimer_end(s);
 }
 
 cudaError_t launch_seed_lift(const PolyDev& P, double lambda0, int64_t N0, int shrink_steps,
@@ -98,14 +85,7 @@ cudaError_t launch_seed_lift(const PolyDev& P, double lambda0, int64_t N0, int s
 cudaError_t launch_walk(const PolyDev& P, double lambda0, int M, int every, int64_t L,
                         int64_t nchunks, const double2* seeds, double2* starts, DevCounters* ctr,
                         cudaStream_t s, int block) {
-  const int bs = (block >= 32 && block <= 1024 && block % 32 == 0) ? block : 64;
-  const int64_t grid = (nchunks + bs - 1) / bs;
-  MT_COUNT_LAUNCH(1);
-  cudaError_t e = ktimer_begin(KS_WALK, s);
-  if (e != cudaSuccess) return e;
-  k_walk<<<(unsigned)grid, bs, 0, s>>>(P, lambda0, M, every, L, nchunks, seeds, starts, ctr);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return ktimer_end(s);
+  return launch_walk_range(P, lambda0, M, every, L, nchunks, 0, nchunks, seeds, starts, ctr, s, block);
 }
 
 // Repairs of the mixed tier in binary64, inside the same launch sequence
@@ -132,24 +112,22 @@ __global__ void k_seed_repair(PolyDev P, double lambda0, int64_t N0, int log2N0,
   warp_add_u64(&ctr->walk_fail, 0ull - fixed);
 }
 
+template <int FB, bool CAP>
 __global__ void k_walk_repair(PolyDev P, double lambda0, int M, int every, int64_t L, int64_t nchunks,
                               int64_t N0, int log2N0, int shrink, const double2* __restrict__ seeds,
                               double2* __restrict__ starts, uint8_t* __restrict__ chunk_fail,
                               DevCounters* ctr, int64_t j0, int64_t nch) {
   __shared__ double2 ph[64];
-  for (int q = threadIdx.x; q < M; q += blockDim.x) {
-    double c, s;
-    unit_phase((uint64_t)q, (uint64_t)M, c, s);
-    ph[q] = make_double2(lambda0 * c, lambda0 * s);
-  }
-  __syncthreads();
+  __shared__ longlong2 phx[64];
+  walk_phases<FB>(lambda0, M, ph, phx);
   const int64_t jl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j = j0 + jl;
   unsigned long long steps = 0, fixed = 0;
   if (jl < nch && j < nchunks && chunk_fail[j]) {
     const double2 a = lift_seed(P, lambda0, N0, log2N0, shrink, j, steps);
     const double2 b = lift_seed(P, lambda0, N0, log2N0, shrink, j + 1, steps);
-    if (!walk_chunk_from(P, ph, M, every, L, nchunks, j, a, b, starts, steps, j0 * L / every)) {
+    if (!walk_chunk_from<FB, CAP>(P, lambda0, M, every, L, nchunks, j, a, b, ph, phx, starts, steps,
+                                  j0 * L / every)) {
       chunk_fail[j] = 0;
       fixed = 1;
     }
@@ -179,8 +157,13 @@ cudaError_t launch_mixed_repair_walk(const PolyDev& P, double lambda0, int M, in
   const int64_t N0 = 2 * nchunks;
   int log2N0 = 0;
   while ((int64_t(1) << log2N0) < N0) ++log2N0;
+  const int fb = walk_fb(P, lambda0);
+  const bool cap = P.lcap >= 1;
+  const auto kern = fb == 28 ? (cap ? &k_walk_repair<28, true> : &k_walk_repair<28, false>)
+                    : fb == 26 ? (cap ? &k_walk_repair<26, true> : &k_walk_repair<26, false>)
+                               : (cap ? &k_walk_repair<0, true> : &k_walk_repair<0, false>);
   MT_COUNT_LAUNCH(1);
-  k_walk_repair<<<(unsigned)((nch + 127) / 128), 128, 0, s>>>(P, lambda0, M, every, L, nchunks, N0, log2N0,
+  kern<<<(unsigned)((nch + 127) / 128), 128, 0, s>>>(P, lambda0, M, every, L, nchunks, N0, log2N0,
                                                               shrink, seeds, starts, chunk_fail, ctr, j0, nch);
   return cudaGetLastError();
 }

@@ -29,6 +29,7 @@
 // its binary64 finishing steps.  The chunk-end check of the walk and the
 // count check catch any tracking failure, and the host then repeats the
 // split in plain binary64.
+#include "mt_ff.cuh"
 #include "mt_levelline.cuh"
 #include "mt_pert.cuh"
 
@@ -36,38 +37,6 @@ namespace mt {
 
 constexpr int MIX_MAXM = 41;
 constexpr int64_t MIX_BATCH = int64_t(1) << 23;  // starts per launch of the binary32 descent
-
-// Float-float (binary32 pair) arithmetic from the published error-free
-// transforms: Knuth's TwoSum, Dekker's FastTwoSum and the FMA-based TwoProd.
-// ~48-bit accurate; used where a binary64 result is not needed but binary32
-// is not enough (the descents' anchor orbits).
-struct ff { float hi, lo; };
-
-__device__ __forceinline__ ff ff_from(double x) {
-  ff r;
-  r.hi = (float)x;
-  r.lo = (float)(x - (double)r.hi);
-  return r;
-}
-__device__ __forceinline__ ff ff_norm(float s, float e) {  // FastTwoSum, |s| >= |e|
-  ff r;
-  r.hi = s + e;
-  r.lo = e - (r.hi - s);
-  return r;
-}
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-  const float s = a.hi + b.hi;  // TwoSum
-  const float bb = s - a.hi;
-  const float e = (a.hi - (s - bb)) + (b.hi - bb) + (a.lo + b.lo);
-  return ff_norm(s, e);
-}
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-  const float p = a.hi * b.hi;  // TwoProd
-  const float e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)));
-  return ff_norm(p, e);
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return ff{-a.hi, -a.lo}; }
-__device__ __forceinline__ ff ff_twice(ff a) { return ff{a.hi + a.hi, a.lo + a.lo}; }
 
 // binary64 reference orbit at c0: zs[k * stride] = Z_k in binary32 for
 // k = 0 .. m-1 (truncated on the integer pipe: the binary64 pipe keeps the

@@ -5,6 +5,10 @@
 // iterate jumps far away (a long-distance jump, Sec. 6.4.1), or the cap
 // max{20, I_N log2 d} of Algorithm S_par is reached.
 //
+// p_n and s_{l,n} descend in 64-bit fixed point on the integer pipes
+// (mt_descent.cuh, mt_fix.cuh); q_{l,n}, whose product form has no such bound
+// on its values, in binary64.
+//
 // GB300 design.  Descent lengths vary (about 10-12 steps when convergent,
 // the cap when not; Sec. 6.4.1), which is the paper's own objection to a
 // GPU port (Sec. 6.4.5: lock-step lanes would make the worst case the
@@ -12,15 +16,16 @@
 // drains one atomic work queue; a lane that finishes its descent is refilled
 // at the next step through a warp vote (__ballot_sync) and one atomicAdd per
 // warp, so lanes never idle while the queue holds work.
-#include "mt_common.cuh"
+#include "mt_descent.cuh"
 
 namespace mt {
 
 // LIST: the starts list[0 .. *nlist) only (start list[t] for queue entry
-// t); the queue is ctr->queue_head2 then.
-template <bool LIST>
+// t); the queue is ctr->queue_head2 then.  CAP: P has a captured term
+// (s_{l,n}).
+template <bool LIST, bool CAP>
 __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __restrict__ starts,
-                                                 int64_t count, double tol2, int cap,
+                                                 int64_t count, float tol2, int cap,
                                                  double2* __restrict__ cand,
                                                  uint8_t* __restrict__ status, DevCounters* ctr,
                                                  const uint32_t* __restrict__ list = nullptr,
@@ -30,63 +35,51 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
   const unsigned lane = threadIdx.x & 31;
   int64_t idx = -1;  // current queue entry (-1: idle, >= count: queue drained)
   int64_t at = 0;    // its start
-  double zr = 0.0, zi = 0.0, rdiv2 = 16.0, prev2 = 1e300;
-  int it = 0;
-  unsigned long long steps = 0, nconv = 0, ndiv = 0, nto = 0;
+  int outcome = -1;  // of the lane's finished descent, until it is written
+  Descent d{0, 0, 16.f, 3.0e38f, 0, false, true};
+  unsigned steps = 0, nconv = 0, ndiv = 0, nto = 0;
+  bool drained = false;  // warp-uniform
   for (;;) {
-    // refill idle lanes from the queue (one atomic per warp)
-    const unsigned need = __ballot_sync(0xffffffffu, idx < 0);
-    if (need) {
-      unsigned long long base = 0;
-      if (lane == (unsigned)(__ffs(need) - 1)) base = atomicAdd(queue, (unsigned long long)__popc(need));
-      base = __shfl_sync(0xffffffffu, base, __ffs(need) - 1);
-      if (idx < 0) {
-        idx = (int64_t)(base + __popc(need & lanemask_lt()));
-        if (idx < count) {
-          at = LIST ? (int64_t)list[idx] : idx;
-          const double2 z0 = starts[at];
-          zr = z0.x;
-          zi = z0.y;
-          it = 0;
-          prev2 = 1e300;
-          // long jump: beyond twice the start radius and outside D(0, 4)
-          rdiv2 = fmax(16.0, 4.0 * fma(zr, zr, zi * zi));
-        }
-      }
-    }
-    const bool active = idx >= 0 && idx < count;
-    if (!__any_sync(0xffffffffu, active)) break;
-    if (active) {
-      double vr, vi, dr, di;
-      eval_P(P, zr, zi, vr, vi, dr, di);
-      double qr, qi;
-      cdiv_f64(vr, vi, dr, di, qr, qi);
-      zr -= qr;
-      zi -= qi;
-      ++it;
-      ++steps;
-      const double s2 = fma(qr, qr, qi * qi);
-      int outcome = -1;
-      // Past the finiteness test z, hence q, is finite, so |z|^2, s2, rdiv2,
-      // tol2 and prev2 are all in [+0, +inf], and prev2 >= tol2 >= 1e-300 (a
-      // step below tol2 ends the descent): they compare as integers
-      // (s2 >= prev2 / 4 as ord(s2) >= ord(prev2) - ORD_QUARTER).
-      if (!finite2(zr, zi) || ord_f64(fma(zr, zr, zi * zi)) > ord_f64(rdiv2)) outcome = 1;
-      else if (ord_f64(s2) < ord_f64(tol2)) outcome = 0;  // the step that met tol also squared the error
-      // binary64 rounding floor: steps stopped shrinking within a few ulp of z
-      // (between two close roots Newton also stalls, at |step| ~ their
-      // separation^2 / distance, far above this floor)
-      else if (ord_f64(s2) >= ord_f64(prev2) - ORD_QUARTER && s2 < floor2_f64(zr, zi)) outcome = 0;
-      else if (it >= cap) outcome = 2;
-      prev2 = s2;
+    // Lanes that finished are written and refilled together, once DESC_REFILL
+    // of them wait or none is running: both cost a pass of the warp however
+    // few lanes take it (one atomic per warp).
+    const bool active0 = idx >= 0 && idx < count && outcome < 0;
+    const unsigned running = __ballot_sync(0xffffffffu, active0);
+    const unsigned wait = __popc(__ballot_sync(0xffffffffu, idx < 0 || outcome >= 0));
+    if (wait >= DESC_REFILL || running == 0u) {
       if (outcome >= 0) {
-        cand[at] = make_double2(zr, zi);
+        cand[at] = descent_point(d);
         status[at] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
         nto += outcome == 2;
+        outcome = -1;
         idx = -1;
       }
+      const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
+      if (need) {
+        unsigned long long base = 0;
+        if (lane == (unsigned)(__ffs(need) - 1)) base = atomicAdd(queue, (unsigned long long)__popc(need));
+        base = __shfl_sync(0xffffffffu, base, __ffs(need) - 1);
+        drained = (int64_t)(base + __popc(need)) >= count;
+        if (idx < 0) {
+          idx = (int64_t)(base + __popc(need & lanemask_lt()));
+          if (idx < count) {
+            at = LIST ? (int64_t)list[idx] : idx;
+            descent_start(d, starts[at], P.fx != 0);
+          }
+        }
+      }
+      if (drained && idx < 0) idx = count;
+    }
+    const bool active = idx >= 0 && idx < count && outcome < 0;
+    if (!__any_sync(0xffffffffu, active)) {
+      if (drained && !__any_sync(0xffffffffu, outcome >= 0)) break;
+      continue;
+    }
+    if (active) {
+      outcome = descent_step<CAP>(P.m, P.lcap, d, tol2, cap);
+      ++steps;
     }
   }
   warp_add_u64(&ctr->desc_newton, steps);
@@ -286,15 +279,17 @@ cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t coun
   const int bs = 128;
   (void)block;
   int per_sm = 0;
+  const auto kd = P.lcap >= 1 ? &k_descend<false, true> : &k_descend<false, false>;
   cudaError_t e = P.kind == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_descend_q, bs, 0)
-                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_descend<false>, bs, 0);
+                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kd, bs, 0);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
-  // The binary64 pipe (2 DFMA lanes per SM on GB300) is saturated by 8 warps
-  // per SM; more resident lanes only lengthen the tail in which a warp waits
-  // for its last descents.  Measured at p_20: 10 blocks/SM 4.18 ms, 4 blocks
-  // 3.76 ms, 2 blocks 3.56 ms, 1 block 3.88 ms.
-  if (per_sm > 2) per_sm = 2;
+  // p_n, s_{l,n} (integer pipes): 24 warps per SM hide the multiply-adds'
+  // latency; more only lengthen the tail in which a warp waits for its last
+  // descents.  Measured: p_20 3 blocks 0.89 ms, 4 0.85, 5 0.84, 6 0.84, 8
+  // 0.87; p_24 15.6, 14.4, 13.9, 13.6, 13.4.
+  // q_{l,n} (binary64 pipe, 2 lanes per SM): saturated by 8 warps per SM.
+  if (per_sm > (P.kind == 2 ? 2 : 6)) per_sm = P.kind == 2 ? 2 : 6;
   int64_t grid = (int64_t)device_sm_count() * per_sm;
   const int64_t need = (count + bs - 1) / bs;
   if (grid > need) grid = need;
@@ -303,8 +298,7 @@ cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t coun
   if (P.kind == 2)
     k_descend_q<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol * tol, cap, cand, status, ctr);
   else
-    k_descend<false><<<(unsigned)grid, bs, 0, s>>>(P, starts, count, fmax(tol * tol, 1e-300), cap, cand, status,
-                                                   ctr);
+    kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, cand, status, ctr, nullptr, nullptr);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return ktimer_end(s);
 }
@@ -316,9 +310,10 @@ cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const u
   if (P.kind == 2) return cudaErrorInvalidValue;  // q_{l,n} has no mixed tier
   const int bs = 128;
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_descend<true>, bs, 0);
+  const auto kd = P.lcap >= 1 ? &k_descend<true, true> : &k_descend<true, false>;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kd, bs, 0);
   if (e != cudaSuccess) return e;
-  if (per_sm > 2) per_sm = 2;  // as launch_descend
+  if (per_sm > 6) per_sm = 6;  // as launch_descend
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)device_sm_count() * per_sm;
   const int64_t need = (count + bs - 1) / bs;
@@ -326,8 +321,7 @@ cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const u
   if ((e = cudaMemsetAsync(&ctr->queue_head2, 0, sizeof(ctr->queue_head2), s)) != cudaSuccess) return e;
   MT_COUNT_LAUNCH(1);
   if ((e = ktimer_begin(KS_DESC64, s)) != cudaSuccess) return e;
-  k_descend<true><<<(unsigned)grid, bs, 0, s>>>(P, starts, count, fmax(tol * tol, 1e-300), cap, cand, status, ctr,
-                                                list, nlist);
+  kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, cand, status, ctr, list, nlist);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return ktimer_end(s);
 }
