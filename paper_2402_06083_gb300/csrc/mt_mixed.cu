@@ -36,7 +36,6 @@
 namespace mt {
 
 constexpr int MIX_MAXM = 41;
-constexpr int64_t MIX_BATCH = int64_t(1) << 23;  // starts per launch of the binary32 descent
 
 // binary64 reference orbit at c0: zs[k * stride] = Z_k in binary32 for
 // k = 0 .. m-1 (truncated on the integer pipe: the binary64 pipe keeps the
@@ -313,124 +312,275 @@ WalkMixedFn walk_mixed_kernel(const PolyDev& P) {
   return f ? f : &k_walk_mixed<false, 0>;
 }
 
-// a4 in the mixed tier, anchors: the reference orbit of a start c0 in
-// float-float, rounded to binary32 (Z_k, k = 1 .. m-1), plus P(c0) as
-// binary32 hi + lo and the long-jump bound on |delta|.  The anchor only
-// steers the binary32 descent into the basin of its root (the binary64
-// finish sets the digits), so float-float's ~1e-14 suffices and keeps this
-// off the binary64 pipe.  A warp computes the orbits of the 32 starts of a
-// queue range together, lane j the orbit of start g + j, into its own slot
-// of the buffer: Z_k of lane j at za[(k - 1) * 32 + j] (each store
-// instruction writes 256 contiguous bytes), P(c0) at zv[j], the bound at
-// zr[j].  The slots are small (32 orbits per warp) and are read back by the
-// same warp moments later, so they stay in L2.
+// a4 in the mixed tier, anchors.  One reference orbit serves the descents of
+// 2^gsh consecutive starts of the line (a turn for 4): the orbit of one of
+// them, c0, in float-float, rounded to binary32 (Z_k), plus P(c0) as binary32
+// hi + lo and the long-jump bound on |delta|.  The anchor only steers the
+// binary32 descent into the basin of its root (the binary64 finish sets the
+// digits), so float-float's ~1e-14 suffices and keeps this off the binary64
+// pipe.
+//
+// The first K orbit steps of every Newton step are replaced by the cubic of
+// p_K around c0: e_K = A d + B d^2 + C d^3 with A = p'_K, B = p''_K / 2, C =
+// p^(3)_K / 6 at c0, carried along the anchor's orbit (A' = 2 Z A + 1, B' =
+// 2 Z B + A^2, C' = 2 Z C + 2 A B).  e grows about twofold a step, to ~|P| at
+// the end, so it is still small at K = m - DM_TAIL, where the dropped fourth
+// term is 1e-6 of e inside |d| <= rho, |C| rho^2 = 1e-4 |A| and |B| rho =
+// 1e-2 |A| (deep-zoom renderers' series approximation).  At p_28 the median
+// descent needs 9 steps after the series, nine in ten 12.
+//
+// A warp computes the orbits of a queue range together, lane j the one of
+// the j-th group, into its own slot of the buffer: Z_k of lane j at
+// za[(k - K) * 32 + j] (each store instruction writes 256 contiguous bytes).
+// The slots are small and are read back by the same warp moments later, so
+// they stay in L2.
 struct WarpSlot {
-  float2* za;  // [m - 1][32]
-  float4* zv;  // [32]
-  float* zr;   // [32]
+  float2* za;   // [m - K][32]
+  float4* zv;   // [32] P(c0)
+  float4* zab;  // [32] A, B
+  float4* zcr;  // [32] C, rho^2, long-jump bound
+  double2* c0;  // [32]
 };
-__device__ __forceinline__ WarpSlot warp_slot(float2* wbuf, int m1, unsigned warp) {
-  const size_t per = (size_t)32 * m1 + 80;  // float2 units: anchors, 32 float4, 32 float
+constexpr int SLOT_EXTRA = 32 * 8;  // float2 units of the four small arrays
+__device__ __forceinline__ WarpSlot warp_slot(float2* wbuf, int rows, unsigned warp) {
+  const size_t per = (size_t)32 * rows + SLOT_EXTRA;  // float2 units
   float2* b = wbuf + per * warp;
   WarpSlot w;
-  w.za = b;
-  w.zv = (float4*)(b + (size_t)32 * m1);
-  w.zr = (float*)(b + (size_t)32 * m1 + 64);
+  w.c0 = (double2*)b;
+  w.zv = (float4*)(b + 64);
+  w.zab = (float4*)(b + 128);
+  w.zcr = (float4*)(b + 192);
+  w.za = b + SLOT_EXTRA;
   return w;
 }
 template <bool CAP, int MC>
-__device__ __forceinline__ void anchor_orbit(const PolyDev& P, double2 c0, const WarpSlot& w, unsigned j) {
+__device__ __forceinline__ void anchor_orbit(const PolyDev& P, int K, double2 c0, const WarpSlot& w, unsigned j) {
   const int m = MC > 0 ? MC : P.m;
   const ff cx = ff_from(c0.x), cy = ff_from(c0.y);
-  ff zx{0.f, 0.f}, zy{0.f, 0.f}, capx{0.f, 0.f}, capy{0.f, 0.f};
-#pragma unroll 4
-  for (int k = 1; k <= m; ++k) {
+  ff zx = cx, zy = cy, capx{0.f, 0.f}, capy{0.f, 0.f};  // Z_1 = c0
+  if (CAP && P.lcap == 1) { capx = zx; capy = zy; }
+  float Ax = 1.f, Ay = 0.f, Bx = 0.f, By = 0.f, Cx = 0.f, Cy = 0.f;
+  auto next = [&](int k) {  // Z_k -> Z_{k+1}
     const ff nx = ff_add(ff_add(ff_mul(zx, zx), ff_neg(ff_mul(zy, zy))), cx);
     const ff ny = ff_add(ff_twice(ff_mul(zx, zy)), cy);
     zx = nx;
     zy = ny;
-    if (k < m) w.za[(k - 1) * 32 + j] = make_float2(zx.hi, zy.hi);
-    if (CAP && k == P.lcap) { capx = zx; capy = zy; }
+    if (CAP && k + 1 == P.lcap) { capx = zx; capy = zy; }
+  };
+#pragma unroll 2
+  for (int k = 1; k < K; ++k) {
+    const float tx = zx.hi + zx.hi, ty = zy.hi + zy.hi;
+    const float nCx = fmaf(tx, Cx, fmaf(-ty, Cy, 2.f * fmaf(Ax, Bx, -Ay * By)));
+    const float nCy = fmaf(tx, Cy, fmaf(ty, Cx, 2.f * fmaf(Ax, By, Ay * Bx)));
+    const float nBx = fmaf(tx, Bx, fmaf(-ty, By, fmaf(Ax, Ax, -Ay * Ay)));
+    const float nBy = fmaf(tx, By, fmaf(ty, Bx, 2.f * Ax * Ay));
+    const float nAx = fmaf(tx, Ax, fmaf(-ty, Ay, 1.f));
+    const float nAy = fmaf(tx, Ay, ty * Ax);
+    Ax = nAx; Ay = nAy; Bx = nBx; By = nBy; Cx = nCx; Cy = nCy;
+    next(k);
+  }
+#pragma unroll 4
+  for (int k = K; k < m; ++k) {
+    w.za[(k - K) * 32 + j] = make_float2(zx.hi, zy.hi);
+    next(k);
   }
   const ff vx = ff_add(zx, capx), vy = ff_add(zy, capy);
   w.zv[j] = make_float4(vx.hi, vy.hi, vx.lo, vy.lo);
+  // rho^2; no bound where nothing is skipped, 0 (never valid) out of binary32's range
+  float rho2 = 3.0e38f;
+  if (K > 1) {
+    const float a = fmaf(Ax, Ax, Ay * Ay), b = fmaf(Bx, Bx, By * By), c = sqrtf(fmaf(Cx, Cx, Cy * Cy));
+    rho2 = fminf(1e-4f * sqrtf(a) / c, 1e-4f * a / b);
+    if (!(c < 1e37f && b < 1e37f && rho2 > 0.f)) rho2 = 0.f;
+  }
   // long jump (as in k_descend: |c| > max(4, 2|c0|)); |delta| beyond rdel implies it
   const float r0 = sqrtf(fmaf(cx.hi, cx.hi, cy.hi * cy.hi)) * 1.0001f;
-  w.zr[j] = fmaxf(4.f, 2.f * r0) + r0;
+  w.zab[j] = make_float4(Ax, Ay, Bx, By);
+  w.zcr[j] = make_float4(Cx, Cy, rho2, fmaxf(4.f, 2.f * r0) + r0);
+  w.c0[j] = c0;
+}
+
+// Newton quotient's e and D = P'(c0 + d) from the series at K and the orbit
+// steps K .. m-1; z1 points to Z_K of the lane's column.
+template <bool CAP, int MC, int KC, int STRIDE>
+__device__ __forceinline__ void pert_eval_series(const PolyDev& P, int Kr, const float2* z1, const float4& ab, float cx,
+                                                 float cy, float dx, float dy, float& ex, float& ey, float& Dx,
+                                                 float& Dy) {
+  const int m = MC > 0 ? MC : P.m, K = MC > 0 ? KC : Kr;
+  float e_x, e_y, g_x, g_y;
+  if (MC > 0 && KC == 1) {
+    e_x = dx; e_y = dy; g_x = 0.5f; g_y = 0.f;
+  } else {
+    const float d2x = fmaf(dx, dx, -dy * dy), d2y = 2.f * dx * dy;
+    // A + B d + C d^2, and A + 2 B d + 3 C d^2
+    const float bx = fmaf(ab.z, dx, -ab.w * dy), by = fmaf(ab.z, dy, ab.w * dx);
+    const float qx = fmaf(cx, d2x, -cy * d2y), qy = fmaf(cx, d2y, cy * d2x);
+    const float sx = ab.x + (bx + qx), sy = ab.y + (by + qy);
+    e_x = fmaf(sx, dx, -sy * dy);
+    e_y = fmaf(sx, dy, sy * dx);
+    const float h = __int_as_float((127 - K) << 23);  // 2^-K
+    g_x = h * fmaf(3.f, qx, fmaf(2.f, bx, ab.x));
+    g_y = h * fmaf(3.f, qy, fmaf(2.f, by, ab.y));
+  }
+  float ce_x = 0.f, ce_y = 0.f, cg_x = 0.f, cg_y = 0.f;
+  if (CAP && P.lcap == K) { ce_x = e_x; ce_y = e_y; cg_x = g_x; cg_y = g_y; }
+  auto step = [&](int k, float h) {
+    const float2 Z = z1[(k - K) * STRIDE];
+    const float zx = Z.x + e_x, zy = Z.y + e_y;  // p_k(c)
+    const float ng_x = fmaf(zx, g_x, fmaf(-zy, g_y, h));
+    const float ng_y = fmaf(zx, g_y, zy * g_x);
+    const float sx = Z.x + zx, sy = Z.y + zy;  // 2 Z_k + e_k
+    const float ne_x = fmaf(sx, e_x, fmaf(-sy, e_y, dx));
+    const float ne_y = fmaf(sx, e_y, fmaf(sy, e_x, dy));
+    e_x = ne_x; e_y = ne_y; g_x = ng_x; g_y = ng_y;
+    if (CAP && k + 1 == P.lcap) { ce_x = e_x; ce_y = e_y; cg_x = g_x; cg_y = g_y; }
+  };
+  if constexpr (MC > 0) {
+#pragma unroll
+    for (int k = KC; k < MC; ++k) step(k, __int_as_float((126 - k) << 23));  // 2^-(k+1)
+  } else {
+    int hexp = (126 - K) << 23;  // exponent field of 2^-(k+1), k = K
+#pragma unroll 4
+    for (int k = K; k < P.m; ++k) {
+      step(k, __int_as_float(hexp));
+      hexp -= 1 << 23;
+    }
+  }
+  const float sc = __int_as_float((127 + m) << 23);
+  if (CAP) {
+    ex = e_x + ce_x;
+    ey = e_y + ce_y;
+    const float a = P.lcap > 0 ? __int_as_float((127 + P.lcap - m) << 23) : 0.f;
+    Dx = fmaf(a, cg_x, g_x) * sc;
+    Dy = fmaf(a, cg_y, g_y) * sc;
+  } else {
+    ex = e_x;
+    ey = e_y;
+    Dx = g_x * sc;
+    Dy = g_y * sc;
+  }
 }
 
 // a4 in the mixed tier, binary32 phase (persistent, per-lane refill as in
-// k_descend) over starts [base, base + cnt), cnt < 2^31.  Each lane keeps
-// the anchor orbit of its descent (Z_1 .. Z_{m-1}) in its own column of
-// shared memory (row k - 1 holds Z_k of every lane; the row stride DM_BS + 1
-// is odd, so the rows of one column fall in different banks).  Lanes that
-// finished are refilled together once DM_REFILL of them wait (or none is
-// running): they take the next start indices of the warp's range of the
-// work queue, and a refilled lane copies its orbit from the warp's slot
-// into its column (m - 1 independent loads, L2 hits).  When the range runs
-// out the warp takes the next one (one atomic per 32 starts) and computes
-// its 32 anchor orbits with every lane (anchor_orbit): the orbits cost one
-// full-width pass per 32 starts and never travel through HBM.  The Newton
-// loop is binary32 only.  Each descent runs binary32 Newton steps to the
-// binary32 floor and leaves (delta, its largest squared step) in pack[]
-// with status 3 ("finish in binary64"), or stops as divergent (1) / timed
-// out (2).  The binary64 finish runs in k_finish_f64, a separate uniform
-// launch, once per root.  MC: the orbit length when fixed at compile time
-// (p_n), else 0.
-constexpr int DESC_POOL = 32;  // work indices taken per queue atomic (one per lane of a range)
+// k_descend) over starts [0, cnt), or with LIST over list[0 ..
+// *nlist).  Each lane keeps the end of its anchor's orbit (Z_K .. Z_{m-1})
+// in its own column of shared memory (row k - K holds Z_k of every lane; the
+// row stride DM_BS + 1 is odd, so the rows of one column fall in different
+// banks).  Lanes that finished are refilled together once DM_REFILL of them
+// wait (or none is running): they take the next start indices of the warp's
+// range of the work queue, and a refilled lane copies its orbit from the
+// warp's slot into its column (m - K independent loads, L2 hits).  When the
+// range (32 groups of 2^gsh starts) runs out the warp takes the next one (one
+// atomic) and computes its 32 anchor orbits with every lane (anchor_orbit):
+// the orbits cost one full-width pass per 32 2^gsh starts and never travel
+// through HBM.  The Newton loop is binary32 only.  Each descent runs binary32
+// Newton steps to the binary32 floor and leaves (delta from its start, its
+// largest squared step) in pack[] with status 3 ("finish in binary64"), or
+// stops as divergent (1) / timed out (2).  One that leaves the series' radius
+// goes on the far list with its state (status 5) and is continued there
+// without a series (LIST, K = 1, its own start as the anchor), so that no warp
+// runs the whole orbit for one of its lanes.  MC: the orbit length when fixed
+// at compile time (p_n), else 0.
+//
+// Bound by issue (80 %) and the binary32 pipe (50 %).  p_28, 268 M starts: 53.4
+// ms with an anchor a start and every orbit step, 29.1 now; p_24 2.93 -> 1.84.
 constexpr int DM_BS = 128;     // threads per block of the binary32 descent
-constexpr int DM_REFILL = 4;   // idle lanes that trigger a refill
+// Idle lanes that trigger a refill, and orbit steps after the series: the
+// refill's pass (the end's record, the next orbit's copy) costs about a third of a
+// Newton step.  p_28, ms of the kernel: 4 lanes 31.7, 6 30.1, 8 29.5, 11 29.1 at 12
+// steps; 10 / 14 / 16 steps +5.0 / -0.3 / +0.5 at 4 lanes, 14 +0.3 at 8.
+constexpr int DM_REFILL = 11;
 constexpr int DM_MAX_WARPS = 16384;  // warp slots of the anchor buffer (grids are capped to fit)
+constexpr int DM_TAIL = 12;
+// Orbits shorter than this run whole: the skipped steps no longer pay for the far
+// list's launch (p_16: 0.061 ms whole, 0.079 with 4 steps skipped; p_20 0.183 and 0.182).
+constexpr int DM_SERIES_MIN = 20;
 
-template <bool CAP, int MC>
-__global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, const double2* __restrict__ starts,
-                                                         int64_t base, int64_t cnt, float2* wbuf, int cap,
-                                                         float4* __restrict__ pack,
-                                                         uint8_t* __restrict__ status,
-                                                         unsigned* queue, DevCounters* ctr) {
+template <bool CAP, int MC, bool LIST>
+__global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, int Kr, int gsh,
+                                                         const double2* __restrict__ starts, int64_t cnt,
+                                                         float2* wbuf, int cap, float4* __restrict__ pack,
+                                                         uint8_t* __restrict__ status, unsigned* queue,
+                                                         uint32_t* list, unsigned long long* nlist,
+                                                         DevCounters* ctr) {
   extern __shared__ float2 zsh[];
   constexpr int stride = DM_BS + 1;
-  const float2* zs = zsh + threadIdx.x;  // row 0 (Z_1) of this lane's column
+  constexpr int KC = MC >= DM_SERIES_MIN ? MC - DM_TAIL : 1;
+  const int K = MC > 0 ? KC : Kr;
+  const float2* zs = zsh + threadIdx.x;  // row 0 (Z_K) of this lane's column
   const unsigned lane = threadIdx.x & 31;
-  const int m1 = (MC > 0 ? MC : P.m) - 1;
-  const unsigned n = (unsigned)cnt;
-  const WarpSlot ws = warp_slot(wbuf, m1, (blockIdx.x * DM_BS + threadIdx.x) >> 5);
-  unsigned idx = ~0u;  // this lane's start (~0u: none)
-  float dx = 0.f, dy = 0.f, h1 = 0.f, prev2 = 0.f, rdelta = 0.f;
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int rows = (MC > 0 ? MC : P.m) - K;
+  const unsigned n = LIST ? (unsigned)*nlist : (unsigned)cnt;
+  const unsigned range = 32u << gsh;  // starts of a queue range
+  const WarpSlot ws = warp_slot(wbuf, rows, (blockIdx.x * DM_BS + threadIdx.x) >> 5);
+  unsigned idx = ~0u;  // this lane's start in the queue (~0u: none)
+  unsigned at = 0;     // its index in starts
+  float dx = 0.f, dy = 0.f, h1 = 0.f, prev2 = 0.f, rdelta = 0.f, d0x = 0.f, d0y = 0.f, rho2 = 0.f, Cx = 0.f, Cy = 0.f;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f), ab = v;
   int it = 0;
-  unsigned long long s32 = 0, ndiv = 0, nto = 0;
-  // the warp's range [pool_base, pool_base + 32) and its next unused index
+  unsigned s32 = 0, ndiv = 0, nto = 0;
+  // the warp's range [pool_base, pool_base + range) and its next unused index
   // (warp-uniform; none taken yet: pool_next at the range's end)
-  unsigned pool_base = 0, pool_next = DESC_POOL;
+  unsigned pool_base = 0, pool_next = range;
   bool drained = false;                   // the queue is empty (warp-uniform)
   // a refilled lane with start i of the range in the slot: its orbit into
   // its column, and the state of a new descent
   auto take_orbit = [&](unsigned i) {
-    const unsigned j = i - pool_base;
+    const unsigned j = (i - pool_base) >> gsh;
     float2* dst = zsh + threadIdx.x;
     if (MC > 0) {
 #pragma unroll
-      for (int k = 0; k < (MC > 0 ? MC - 1 : 1); ++k) dst[k * stride] = ws.za[k * 32 + j];
+      for (int k = 0; k < (MC > 0 ? MC - KC : 1); ++k) dst[k * stride] = ws.za[k * 32 + j];
     } else {
-      for (int k = 0; k < m1; ++k) dst[k * stride] = ws.za[k * 32 + j];
+      for (int k = 0; k < rows; ++k) dst[k * stride] = ws.za[k * 32 + j];
     }
     v = ws.zv[j];
-    rdelta = ws.zr[j];
-    dx = dy = 0.f;
-    it = 0;
-    prev2 = 0.f;
-    h1 = 0.f;
+    ab = ws.zab[j];
+    const float4 cr = ws.zcr[j];
+    Cx = cr.x;
+    Cy = cr.y;
+    rho2 = cr.z;
+    rdelta = cr.w;
+    at = LIST ? list[i] : i;
+    if (LIST) {  // go on from where the series ended
+      const float4 q = pack[at];
+      dx = q.x;
+      dy = q.y;
+      h1 = q.z;
+      it = __float_as_int(q.w);
+      prev2 = 3.0e38f;
+      d0x = d0y = 0.f;
+    } else {
+      const double2 s0 = starts[at], c0 = ws.c0[j];
+      d0x = f32_trunc(s0.x - c0.x);  // exact differences, zero for the anchor itself
+      d0y = f32_trunc(s0.y - c0.y);
+      dx = d0x;
+      dy = d0y;
+      it = 0;
+      prev2 = 0.f;
+      h1 = 0.f;
+    }
   };
+  int outcome = 0;  // >= 0: the lane has no running descent (its last one ended so)
   for (;;) {
-    const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx == ~0u);
-    const unsigned R = __popc(need);
-    if (R >= DM_REFILL || (R == 32u && need)) {
+    const unsigned wait = __ballot_sync(0xffffffffu, outcome >= 0);
+    // write the ended descents and refill their lanes together
+    if (__popc(wait) >= (drained ? 32 : DM_REFILL)) {
+      if (outcome >= 0 && idx < n) {
+        pack[at] = make_float4(dx - d0x, dy - d0y, h1, __int_as_float(it));
+        status[at] = (uint8_t)outcome;
+        ndiv += outcome == 1;
+        nto += outcome == 2;
+        if (!LIST && outcome == 5) list[atomicAdd(nlist, 1ull)] = at;
+        idx = ~0u;
+      }
+      if (drained) break;
+      const unsigned R = __popc(wait);
       // the r-th lane that needs a start takes the r-th unused index of the
       // range, then of the next range
-      const bool mine = (need >> lane) & 1u;
-      const unsigned r_me = __popc(need & lanemask_lt());
-      const unsigned rem = pool_base + DESC_POOL - pool_next;
+      const bool mine = outcome >= 0;
+      const unsigned r_me = __popc(wait & lanemask_lt());
+      const unsigned rem = pool_base + range - pool_next;
       if (mine && r_me < rem) {
         idx = pool_next + r_me;
         if (idx < n) take_orbit(idx);
@@ -440,9 +590,14 @@ __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, const double
       } else {
         __syncwarp();  // the copies above have read the slot
         unsigned g = 0;
-        if (lane == 0) g = atomicAdd(queue, (unsigned)DESC_POOL);
+        if (lane == 0) g = atomicAdd(queue, range);
         g = __shfl_sync(0xffffffffu, g, 0);
-        if (g + lane < n) anchor_orbit<CAP, MC>(P, starts[base + g + lane], ws, lane);
+        // the group's anchor: its middle start (of those that exist)
+        const unsigned first = g + (lane << gsh);
+        if (first < n) {
+          const unsigned a = min(first + ((1u << gsh) >> 1), n - 1u);
+          anchor_orbit<CAP, MC>(P, K, starts[LIST ? list[a] : a], ws, lane);
+        }
         __syncwarp();  // the slot is written before any lane reads it
         pool_base = g;
         pool_next = g + (R - rem);
@@ -451,41 +606,33 @@ __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, const double
           if (idx < n) take_orbit(idx);
         }
       }
-      if (mine && idx >= n) idx = n;  // the queue is drained: never refilled again
-      if (__any_sync(0xffffffffu, mine && idx == n)) drained = true;
+      // the queue is drained once a lane's index lies past its end
+      if (mine) outcome = idx < n ? -1 : 0;
+      drained = __any_sync(0xffffffffu, mine && idx >= n);
     }
-    const bool active = idx < n;
-    if (!__any_sync(0xffffffffu, active)) {
-      if (drained) break;
-      continue;  // every lane idle: the next pass refills all 32
-    }
-    if (active) {
-      int outcome = -1;
+    if (outcome < 0) {
       float ex, ey, Dx, Dy, qr, qi;
-      pert_eval_t<CAP, MC, stride>(P, zs, dx, dy, ex, ey, Dx, Dy);
-      const float nr = (v.x + v.z) + ex, ni = (v.y + v.w) + ey;
-      if (!cdiv_f32(nr, ni, Dx, Dy, qr, qi)) {
-        outcome = 3;  // out of binary32 range: binary64 decides
+      if (!LIST && !(fmaf(dx, dx, dy * dy) <= rho2)) {
+        outcome = 5;  // beyond the series: continued on the far list
       } else {
-        dx -= qr;
-        dy -= qi;
-        ++it;
-        ++s32;
-        const float s2 = fmaf(qr, qr, qi * qi);
-        h1 = fmaxf(h1, s2);  // largest step so far
-        if (!(fmaf(dx, dx, dy * dy) <= rdelta * rdelta)) outcome = 1;
-        // binary32 floor: the step is 1e-5 of the descent's scale, or it
-        // stopped shrinking once already below 1e-3 of it
-        else if (s2 <= 1e-10f * h1 || (s2 <= 1e-6f * h1 && s2 > 0.25f * prev2)) outcome = 3;
-        else if (it >= cap) outcome = 2;
-        prev2 = s2;
-      }
-      if (outcome >= 0) {
-        pack[base + idx] = make_float4(dx, dy, h1, 0.f);
-        status[base + idx] = (uint8_t)outcome;
-        ndiv += outcome == 1;
-        nto += outcome == 2;
-        idx = ~0u;
+        pert_eval_series<CAP, MC, KC, stride>(P, K, zs, ab, Cx, Cy, dx, dy, ex, ey, Dx, Dy);
+        const float nr = (v.x + v.z) + ex, ni = (v.y + v.w) + ey;
+        if (!cdiv_f32(nr, ni, Dx, Dy, qr, qi)) {
+          outcome = 3;  // out of binary32 range: binary64 decides
+        } else {
+          dx -= qr;
+          dy -= qi;
+          ++it;
+          ++s32;
+          const float s2 = fmaf(qr, qr, qi * qi);
+          h1 = fmaxf(h1, s2);  // largest step so far
+          if (!(fmaf(dx, dx, dy * dy) <= rdelta * rdelta)) outcome = 1;
+          // binary32 floor: the step is 1e-5 of the descent's scale, or it
+          // stopped shrinking once already below 1e-3 of it
+          else if (s2 <= 1e-10f * h1 || (s2 <= 1e-6f * h1 && s2 > 0.25f * prev2)) outcome = 3;
+          else if (it >= cap) outcome = 2;
+          prev2 = s2;
+        }
       }
     }
   }
@@ -496,8 +643,8 @@ __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, const double
   warp_add_u64(&ctr->n_timeout, nto);
 }
 
-using DescMixedFn = void (*)(PolyDev, const double2*, int64_t, int64_t, float2*, int, float4*, uint8_t*,
-                             unsigned*, DevCounters*);
+using DescMixedFn = void (*)(PolyDev, int, int, const double2*, int64_t, float2*, int, float4*, uint8_t*, unsigned*,
+                             uint32_t*, unsigned long long*, DevCounters*);
 
 // The instantiation for a polynomial: p_n with 16 <= n <= 33 has its orbit
 // length fixed at compile time; everything else runs the general loop.
@@ -507,13 +654,13 @@ DescMixedFn desc_mixed_fixed(int m) {
     (void)m;
     return nullptr;
   } else {
-    return m == MC ? &k_descend_mixed<false, MC> : desc_mixed_fixed<MC - 1>(m);
+    return m == MC ? &k_descend_mixed<false, MC, false> : desc_mixed_fixed<MC - 1>(m);
   }
 }
 DescMixedFn desc_mixed_kernel(const PolyDev& P) {
-  if (P.lcap >= 0) return &k_descend_mixed<true, 0>;
+  if (P.lcap >= 0) return &k_descend_mixed<true, 0, false>;
   DescMixedFn f = desc_mixed_fixed<33>(P.m);
-  return f ? f : &k_descend_mixed<false, 0>;
+  return f ? f : &k_descend_mixed<false, 0, false>;
 }
 
 // a4 in the mixed tier, binary64 finish, once per root.
@@ -899,42 +1046,62 @@ cudaError_t launch_walk_mixed(const PolyDev& P, double lambda0, int M, int every
 size_t mixed_anchor_bytes(const PolyDev& P, int64_t count) {
   (void)count;
   const int m1 = P.m > 1 ? P.m - 1 : 1;
-  return (size_t)DM_MAX_WARPS * ((size_t)32 * m1 + 80) * sizeof(float2) + 256;
+  return (size_t)DM_MAX_WARPS * ((size_t)32 * m1 + SLOT_EXTRA) * sizeof(float2) + 256;
+}
+
+// One launch of the binary32 descent over starts [0, count), or over the far
+// list (list != nullptr with LIST kernels).
+static cudaError_t launch_dm(DescMixedFn kern, const PolyDev& P, int K, int gsh, const double2* starts, int64_t count,
+                             float2* wbuf, int cap, float4* pack, uint8_t* status, uint32_t* list,
+                             unsigned long long* nlist, DevCounters* ctr, cudaStream_t s) {
+  const int bs = DM_BS;
+  const size_t smem = (size_t)std::max(1, P.m - K) * (bs + 1) * sizeof(float2);
+  cudaError_t e = cudaSuccess;
+  if (smem > 48 * 1024 &&  // long orbits: opt in to more than 48 KB
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, bs, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) per_sm = 1;
+  int64_t grid = (int64_t)device_sm_count() * per_sm;
+  const int64_t need = (count + bs - 1) / bs;
+  if (grid > need) grid = need;
+  if (grid > DM_MAX_WARPS / (bs / 32)) grid = DM_MAX_WARPS / (bs / 32);
+  unsigned* q = (unsigned*)&ctr->queue_head;  // 32 bits: the last ranges end below 2^32
+  if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess) return e;
+  MT_COUNT_LAUNCH(1);
+  if ((e = ktimer_begin(KS_DESC32, s)) != cudaSuccess) return e;
+  kern<<<(unsigned)grid, bs, smem, s>>>(P, K, gsh, starts, count, wbuf, cap, pack, status, q, list, nlist, ctr);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return ktimer_end(s);
 }
 
 cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t count, double tol, int cap,
                                  double2* cand, uint8_t* status, void* anchors, const FinishScratch& fin,
                                  DevCounters* ctr, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
-  if (P.m > MIX_MAXM) return cudaErrorInvalidValue;
+  if (P.m > MIX_MAXM || count > 0xfff00000ll) return cudaErrorInvalidValue;  // 32-bit queue and list
   const int bs = DM_BS;
-  const size_t smem = (size_t)(P.m > 1 ? P.m - 1 : 1) * (bs + 1) * sizeof(float2);
-  const DescMixedFn kdesc = desc_mixed_kernel(P);
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024 &&  // long orbits: opt in to more than 48 KB
-      (e = cudaFuncSetAttribute(kdesc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-    return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kdesc, bs, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
   float2* wbuf = (float2*)anchors;
   float4* pack = (float4*)cand;  // (delta, scale) until the finish writes the roots
-  for (int64_t base = 0; base < count; base += MIX_BATCH) {
-    const int64_t cnt = (count - base < MIX_BATCH) ? count - base : MIX_BATCH;
-    int64_t grid = (int64_t)device_sm_count() * per_sm;
-    const int64_t need = (cnt + bs - 1) / bs;
-    if (grid > need) grid = need;
-    if (grid > DM_MAX_WARPS / (bs / 32)) grid = DM_MAX_WARPS / (bs / 32);
-    // the work queue (32-bit: a batch holds fewer than 2^31 starts) restarts
-    // at 0 for every batch
-    unsigned* q = (unsigned*)&ctr->queue_head;
-    if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess) return e;
-    MT_COUNT_LAUNCH(1);
-    if ((e = ktimer_begin(KS_DESC32, s)) != cudaSuccess) return e;
-    kdesc<<<(unsigned)grid, bs, smem, s>>>(P, starts, base, cnt, wbuf, cap, pack, status, q, ctr);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = ktimer_end(s)) != cudaSuccess) return e;
+  {
+    // s_{l,n} keeps an anchor per start and the whole orbit: its line lies at
+    // |s| = 100, and binary32 relative to a neighbour's delta lost tip roots
+    // (s_{6,12}: none of 7 levels without, 3 with).
+    const bool shared = P.kind == 0;
+    const int K = shared && P.m >= DM_SERIES_MIN ? P.m - DM_TAIL : 1;
+    const int gsh = shared ? 2 : 0;
+    uint32_t* far = fin.pos;  // free until the finish's scan
+    unsigned long long* nfar = fin.nheads;
+    if ((e = cudaMemsetAsync(nfar, 0, sizeof(*nfar), s)) != cudaSuccess) return e;
+    if ((e = launch_dm(desc_mixed_kernel(P), P, K, gsh, starts, count, wbuf, cap, pack, status, far, nfar, ctr, s)) !=
+        cudaSuccess)
+      return e;
+    if (K > 1 && (e = launch_dm(&k_descend_mixed<false, 0, true>, P, 1, 0, starts, count, wbuf, cap, pack, status, far,
+                                nfar, ctr, s)) != cudaSuccess)
+      return e;
   }
   // binary64 finish, once per group of end points on the same root
   const unsigned nb = (unsigned)((count + bs - 1) / bs);

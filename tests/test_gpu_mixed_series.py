@@ -1,0 +1,36 @@
+"""The mixed tier's descents on shared anchors and the anchors' series
+(csrc/mt_mixed.cu): orbit lengths on both sides of the rules (general loop
+below 16, fixed lengths from 16, series from 20), starts that do not fill a
+group or a queue range, and denser starts, whose groups span less of a turn."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mt():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2402_06083_gb300 as pkg
+    return pkg
+
+
+@pytest.mark.parametrize("n,kw", [(1, {}), (2, {}), (3, {}), (6, {}), (7, {}), (13, {}), (15, {}), (16, {}), (17, {}),
+                                  (19, {}), (20, {}), (21, {}), (20, {"M": 16, "c_L": 8}), (20, {"M": 8, "c_L": 2}),
+                                  (20, {"lambda0": 5.8}), (18, {"stream_pieces": 4}), (21, {"stream_pieces": 2})])
+def test_first_attempt_finds_every_root(mt, n, kw):
+    """The first attempt alone (no binary64 repeat) is complete and certified,
+    and its roots are the binary64 tier's to the Newton tolerance 1e-13 (each
+    tier stops within it)."""
+    few = kw.get("c_L") == 2  # half the starts: roots are missing, none is wrong
+    r = mt.split_hyperbolic(n, "mixed", max_retries=-1, check_status=not few, **kw)
+    st = r.stats
+    assert st["n_cert_pass"] == st["n_roots"] and st["walk_fail"] == 0
+    if few:
+        return
+    assert st["prec_used"] == 1 and st["n_roots"] == 2 ** (n - 1)
+    a, b = r.roots.cpu().numpy(), mt.split_hyperbolic(n).roots.cpu().numpy()
+    assert np.max(np.abs(a - b)) < 1e-13
