@@ -295,6 +295,209 @@ __global__ void k_walk_mixed(PolyDev P, double lambda0, int M, int every, int64_
   warp_add_u64(&ctr->walk_fail, fails);
 }
 
+// The walk of p_n.  As k_walk_mixed, with fewer and shorter Newton steps:
+//  - The first K orbit steps of each Newton step are the cubic of p_K around
+//    the anchor (as in k_descend_mixed; here within the walk's own tolerance),
+//    K the largest for which it holds within WALK_REACH sub-steps in every
+//    lane of the warp (one vote a step of the anchor's orbit).  The warp
+//    re-anchors early when a lane leaves that radius.
+//  - The predictor extrapolates z' = P / P' along log P from the last three
+//    sub-steps (Adams-Bashforth), and a sub-step that ends on no start stops
+//    once the error left after a correction is small, not once a further
+//    correction has shown it.
+// Bound by issue (70 %) with 14 warps an SM.
+// Shared memory: each warp owns m rows of 32 binary32 pairs.
+constexpr float WALK_REACH = 9.5f;
+
+struct WalkAnchor {
+  float4 v;        // P(c0) as binary32 hi + lo
+  float4 ab;       // A, B at K
+  float cx, cy;    // C at K
+  float rho2;      // the series' radius squared
+  int K;           // warp-uniform
+};
+
+// The anchor's orbit at c0 (binary64) and the series for a reach R.
+__device__ __forceinline__ void walk_anchor(unsigned mask, int m, double px, double py, float R2, float2* zs,
+                                            WalkAnchor& w, double& ax, double& ay) {
+  const ff cx = ff_from(px), cy = ff_from(py);
+  ax = (double)cx.hi + (double)cx.lo;
+  ay = (double)cy.hi + (double)cy.lo;
+  ff zx = cx, zy = cy;
+  float Ax = 1.f, Ay = 0.f, Bx = 0.f, By = 0.f, Cx = 0.f, Cy = 0.f;
+  auto next = [&]() {
+    const ff nx = ff_add(ff_add(ff_mul(zx, zx), ff_neg(ff_mul(zy, zy))), cx);
+    const ff ny = ff_add(ff_twice(ff_mul(zx, zy)), cy);
+    zx = nx;
+    zy = ny;
+  };
+  const float R = sqrtf(R2);
+  w.rho2 = 3.0e38f;
+  int k = 1;
+  for (; k < m - 1; ++k) {
+    const float tx = zx.hi + zx.hi, ty = zy.hi + zy.hi;
+    const float nCx = fmaf(tx, Cx, fmaf(-ty, Cy, 2.f * fmaf(Ax, Bx, -Ay * By)));
+    const float nCy = fmaf(tx, Cy, fmaf(ty, Cx, 2.f * fmaf(Ax, By, Ay * Bx)));
+    const float nBx = fmaf(tx, Bx, fmaf(-ty, By, fmaf(Ax, Ax, -Ay * Ay)));
+    const float nBy = fmaf(tx, By, fmaf(ty, Bx, 2.f * Ax * Ay));
+    const float nAx = fmaf(tx, Ax, fmaf(-ty, Ay, 1.f));
+    const float nAy = fmaf(tx, Ay, ty * Ax);
+    // |C| R^2 <= 6e-3 |A|, |B| R <= 8e-2 |A|: the dropped fourth term is ~5e-4 of
+    // e at the reach, half of a start's tolerance of 1e-2 h
+    const float a1 = fmaxf(fabsf(nAx), fabsf(nAy)), b1 = fmaxf(fabsf(nBx), fabsf(nBy)),
+                c1 = fmaxf(fabsf(nCx), fabsf(nCy));
+    const bool ok = c1 < 1e37f && b1 * R <= 8e-2f * a1 && (c1 * R) * R <= 6e-3f * a1;
+    if (!__all_sync(mask, ok)) break;
+    Ax = nAx; Ay = nAy; Bx = nBx; By = nBy; Cx = nCx; Cy = nCy;
+    next();
+  }
+  w.K = k;
+  if (k > 1) w.rho2 = R2;
+  w.ab = make_float4(Ax, Ay, Bx, By);
+  w.cx = Cx;
+  w.cy = Cy;
+#pragma unroll 2
+  for (; k < m; ++k) {
+    zs[(k - w.K) * 32] = make_float2(zx.hi, zy.hi);
+    next();
+  }
+  w.v = make_float4(zx.hi, zy.hi, zx.lo, zy.lo);
+}
+
+// e_m and D = P' at c0 + d: the series at K, then the orbit steps K .. m-1.
+__device__ __forceinline__ void walk_eval(int m, const WalkAnchor& w, const float2* zs, float dx, float dy, float& ex,
+                                          float& ey, float& Dx, float& Dy) {
+  const float d2x = fmaf(dx, dx, -dy * dy), d2y = 2.f * dx * dy;
+  const float bx = fmaf(w.ab.z, dx, -w.ab.w * dy), by = fmaf(w.ab.z, dy, w.ab.w * dx);
+  const float qx = fmaf(w.cx, d2x, -w.cy * d2y), qy = fmaf(w.cx, d2y, w.cy * d2x);
+  const float tx = w.ab.x + (bx + qx), ty = w.ab.y + (by + qy);
+  float e_x = fmaf(tx, dx, -ty * dy), e_y = fmaf(tx, dy, ty * dx);
+  float h = __int_as_float((127 - w.K) << 23);  // 2^-K
+  float g_x = h * fmaf(3.f, qx, fmaf(2.f, bx, w.ab.x)), g_y = h * fmaf(3.f, qy, fmaf(2.f, by, w.ab.y));
+  auto step = [&](const float2 Z) {
+    h *= 0.5f;
+    const float zx = Z.x + e_x, zy = Z.y + e_y;  // p_k(c)
+    const float ng_x = fmaf(zx, g_x, fmaf(-zy, g_y, h));
+    const float ng_y = fmaf(zx, g_y, zy * g_x);
+    const float sx = Z.x + zx, sy = Z.y + zy;  // 2 Z_k + e_k
+    const float ne_x = fmaf(sx, e_x, fmaf(-sy, e_y, dx));
+    const float ne_y = fmaf(sx, e_y, fmaf(sy, e_x, dy));
+    e_x = ne_x; e_y = ne_y; g_x = ng_x; g_y = ng_y;
+  };
+  const float2* z = zs;
+  const int T = m - w.K;
+  for (int r = T & 3; r > 0; --r, z += 32) step(*z);
+  for (int r = T >> 2; r > 0; --r, z += 128) {
+    step(z[0]);
+    step(z[32]);
+    step(z[64]);
+    step(z[96]);
+  }
+  const float sc = __int_as_float((127 + m) << 23);
+  ex = e_x;
+  ey = e_y;
+  Dx = g_x * sc;
+  Dy = g_y * sc;
+}
+
+__global__ void k_walk_series(PolyDev P, double lambda0, int M, int every, int64_t L, int64_t nchunks, int Kturn,
+                              const double2* __restrict__ seeds, double2* __restrict__ starts,
+                              uint8_t* __restrict__ chunk_fail, DevCounters* ctr, int64_t j0, int64_t nch,
+                              int64_t sbase) {
+  extern __shared__ float2 zsh[];
+  __shared__ float2 ph[64];
+  for (int q = threadIdx.x; q < M; q += blockDim.x) {
+    double c, s;
+    unit_phase((uint64_t)q, (uint64_t)M, c, s);
+    ph[q] = make_float2((float)(lambda0 * c), (float)(lambda0 * s));
+  }
+  __syncthreads();
+  const int m = P.m;
+  float2* zs = zsh + (threadIdx.x >> 5) * 32 * m + (threadIdx.x & 31);
+  const int64_t jl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t j = j0 + jl;
+  unsigned long long steps = 0, fails = 0;
+  const bool mine = jl < nch && j < nchunks;
+  const unsigned mask = __ballot_sync(0xffffffffu, mine);
+  if (mine) {
+    const double2 s0 = seeds[j];
+    double c0x, c0y;
+    WalkAnchor w;
+    walk_anchor(mask, m, s0.x, s0.y, 3.0e37f, zs, w, c0x, c0y);  // no step length yet: the whole orbit
+    float dx = (float)(s0.x - c0x), dy = (float)(s0.y - c0y), h2 = 0.f;
+    bool bad = false;
+    const float Li = 6.2831853f / M;
+    const int esh = __ffs(every) - 1;  // every is a power of two
+    uint64_t g = (uint64_t)j * (uint64_t)L;
+    int kc = 1;  // sub-steps to the next anchor: the first one gives the step length
+    float w1x = 0.f, w1y = 0.f, w2x = 0.f, w2y = 0.f;  // z' at the last two sub-steps
+    for (int64_t i = 0; i < L; ++i, ++g) {
+      if ((g & (uint64_t)(every - 1)) == 0)
+        starts[(int64_t)(g >> esh) - sbase] = make_double2(c0x + (double)dx, c0y + (double)dy);
+      const float2 Tp = ph[g & (uint64_t)(M - 1)];
+      const float2 T = ph[(g + 1) & (uint64_t)(M - 1)];
+      // a correction of r h leaves about r^2 h: r = 1e-2 on the sub-steps that
+      // end on a start (as k_walk_mixed: the roots a line finds depend on its
+      // starts to a few thousandths of a sub-step), r^2 = 1e-1 on the others
+      const float rel2 = (((g + 1) & (uint64_t)(every - 1)) == 0) ? 1e-4f : 1e-1f;
+      float prev2 = 0.f;
+      int it = 0;
+      while (it < 16) {
+        float ex, ey, Dx, Dy, qr, qi;
+        walk_eval(m, w, zs, dx, dy, ex, ey, Dx, Dy);
+        bool ok;
+        if (it == 0) {
+          // -dz = (P - Tp) / P' - L z'_ext, L = i Li, z'_ext = z' and its extrapolation
+          const float Pr = w.v.x + (w.v.z + ex), Pi = w.v.y + (w.v.w + ey);
+          float er, ei, wr, wi;
+          ok = cdiv_f32(((w.v.x - Tp.x) + w.v.z) + ex, ((w.v.y - Tp.y) + w.v.w) + ey, Dx, Dy, er, ei);
+          ok = cdiv_f32(Pr, Pi, Dx, Dy, wr, wi) && ok;
+          float gr = wr, gi = wi;
+          if (i >= 2) {
+            gr = fmaf(1.9166667f, wr, fmaf(-1.3333334f, w1x, 0.41666668f * w2x));
+            gi = fmaf(1.9166667f, wi, fmaf(-1.3333334f, w1y, 0.41666668f * w2y));
+          } else if (i == 1) {
+            gr = fmaf(1.5f, wr, -0.5f * w1x);
+            gi = fmaf(1.5f, wi, -0.5f * w1y);
+          }
+          qr = fmaf(gi, Li, er);
+          qi = fmaf(-gr, Li, ei);
+          w2x = w1x; w2y = w1y;
+          w1x = wr; w1y = wi;
+        } else {
+          ok = cdiv_f32(((w.v.x - T.x) + w.v.z) + ex, ((w.v.y - T.y) + w.v.w) + ey, Dx, Dy, qr, qi);
+        }
+        if (!ok) { bad = true; break; }
+        dx -= qr;
+        dy -= qi;
+        ++it;
+        const float s2 = fmaf(qr, qr, qi * qi);
+        if (it == 1) h2 = s2;
+        else if (s2 <= rel2 * h2 || (it >= 3 && s2 > 0.25f * prev2)) break;
+        prev2 = s2;
+      }
+      steps += it;
+      const bool out = !(fmaf(dx, dx, dy * dy) <= w.rho2 * 0.7f);  // the next sub-step may leave the series
+      if ((--kc == 0 || __any_sync(mask, out)) && i + 1 < L) {  // re-anchor at the current point
+        kc = Kturn;
+        const double px = c0x + (double)dx, py = c0y + (double)dy;
+        walk_anchor(mask, m, px, py, WALK_REACH * WALK_REACH * h2, zs, w, c0x, c0y);
+        dx = (float)(px - c0x);
+        dy = (float)(py - c0y);
+      }
+    }
+    const double cx = c0x + (double)dx, cy = c0y + (double)dy;
+    if (j == nchunks - 1) starts[(int64_t)(g >> esh) - sbase] = make_double2(cx, 0.0);
+    const double2 zn = seeds[j + 1];
+    const double er = cx - zn.x, ei = cy - zn.y;
+    if (bad || !(er * er + ei * ei <= 0.0625 * (double)h2 + 1e-28)) fails = 1;
+    chunk_fail[j] = (uint8_t)fails;  // walked again in binary64 by k_walk_repair
+  }
+  warp_add_u64(&ctr->walk_newton, steps);
+  warp_add_u64(&ctr->steps_fp32, steps);
+  warp_add_u64(&ctr->walk_fail, fails);
+}
+
 using WalkMixedFn = void (*)(PolyDev, double, int, int, int64_t, int64_t, int, const double2*, double2*, uint8_t*,
                              DevCounters*, int64_t, int64_t, int64_t);
 template <int MC>
@@ -306,9 +509,15 @@ WalkMixedFn walk_mixed_fixed(int m) {
     return m == MC ? &k_walk_mixed<false, MC> : walk_mixed_fixed<MC - 1>(m);
   }
 }
+// From p_23 on: below, the line's lanes are too few and the anchors' votes and
+// the loop over a varying length only add latency (ms of the walk, without and
+// with the series: p_20 0.178 and 0.212, p_21 0.222 and 0.246, p_22 0.408 and
+// 0.365, p_24 1.63 and 1.36, p_28 24.9 and 17.8).
+constexpr int WALK_SERIES_MIN = 23;
 WalkMixedFn walk_mixed_kernel(const PolyDev& P) {
   if (P.lcap >= 0) return &k_walk_mixed<true, 0>;
-  WalkMixedFn f = walk_mixed_fixed<33>(P.m);
+  if (P.m >= WALK_SERIES_MIN) return &k_walk_series;
+  WalkMixedFn f = walk_mixed_fixed<WALK_SERIES_MIN - 1>(P.m);
   return f ? f : &k_walk_mixed<false, 0>;
 }
 
@@ -389,9 +598,11 @@ __device__ __forceinline__ void anchor_orbit(const PolyDev& P, int K, double2 c0
   // rho^2; no bound where nothing is skipped, 0 (never valid) out of binary32's range
   float rho2 = 3.0e38f;
   if (K > 1) {
-    const float a = fmaf(Ax, Ax, Ay * Ay), b = fmaf(Bx, Bx, By * By), c = sqrtf(fmaf(Cx, Cx, Cy * Cy));
-    rho2 = fminf(1e-4f * sqrtf(a) / c, 1e-4f * a / b);
-    if (!(c < 1e37f && b < 1e37f && rho2 > 0.f)) rho2 = 0.f;
+    // (in the maximum norm: C ~ A^3 passes 2^64, its square binary32's range)
+    const float a = fmaxf(fabsf(Ax), fabsf(Ay)), b = fmaxf(fabsf(Bx), fabsf(By)), c = fmaxf(fabsf(Cx), fabsf(Cy)),
+                ab = a / b;
+    rho2 = fminf(1e-4f * a / c, 1e-4f * ab * ab);
+    if (!(c < 1e37f && rho2 > 0.f)) rho2 = 0.f;
   }
   // long jump (as in k_descend: |c| > max(4, 2|c0|)); |delta| beyond rdel implies it
   const float r0 = sqrtf(fmaf(cx.hi, cx.hi, cy.hi * cy.hi)) * 1.0001f;
