@@ -395,6 +395,77 @@ __host__ __device__ __forceinline__ void fx_eval(int m, int lcap, int a8, long l
   o.ii = ff_neg(ff_mul(di, r));
 }
 
+#ifdef __CUDACC__
+// w 2^-2FB in binary32, to its full relative precision (two exact halves)
+template <int FB>
+__device__ __forceinline__ float fx_to_f32(long long w) {
+  return fmaf((float)fx_hi(w), fx_pow2f(32 - 2 * FB), (float)(unsigned)w * fx_pow2f(-2 * FB));
+}
+
+// orbit_f64_d32_k (mt_common.cuh) with the value in fixed point: P = (Wr, Wi)
+// 2^-2FB, P' and the curvature P'' / (2 P') in binary32.  False where the
+// orbit leaves the fixed range before its last step.  The value alone is a
+// third of fx_eval's step; its binary32 companions run beside it.
+template <int FB, bool CAP>
+__device__ __forceinline__ bool fx_value_d32_k(int m, int lcap, long long X, long long Y, long long& Wr, long long& Wi,
+                                               float& dr, float& di, float& kr, float& ki) {
+  constexpr int S = 32 - FB;
+  constexpr unsigned R = 1u << (FB - 2);
+  const long long CR = (X + (1ll << (S - 1))) >> S, CI = (Y + (1ll << (S - 1))) >> S;
+  const long long tr0 = ((X - (CR << S)) << (31 - S)) + (1ll << 30);
+  const long long ti0 = ((Y - (CI << S)) << (31 - S)) + (1ll << 30);
+  fx2 x = fx_split(X, 0), y = fx_split(Y, 0);
+  long long wr = CR, wi = CI, cwr = 0, cwi = 0;
+  float dzr = 1.f, dzi = 0.f, capd_r = 0.f, capd_i = 0.f;  // p'_1 = 1, p''_1 = 0
+  float ur = 0.f, ui = 0.f, capu_r = 0.f, capu_i = 0.f;
+  if (CAP && lcap == 1) { cwr = wr; cwi = wi; capd_r = 1.f; }
+  float h = 0.5f;  // 2^-(k-1), k = 2
+  bool in = true;
+#pragma unroll 4
+  for (int k = 2; k <= m; ++k) {
+    const float fr = fx_to_f32<FB>(wr), fi = fx_to_f32<FB>(wi);
+    const float sr = dzr * h, si = dzi * h;  // p'_{k-1} / 2^(k-1)
+    h *= 0.5f;
+    const float nur = 0.5f * (fmaf(sr, sr, -si * si) + fmaf(fr, ur, -fi * ui));
+    const float nui = 0.5f * fmaf(sr + sr, si, fmaf(fr, ui, fi * ur));
+    const float tfr = fr + fr, tfi = fi + fi;
+    const float ndr = fmaf(tfr, dzr, fmaf(-tfi, dzi, 1.f));
+    const float ndi = fmaf(tfr, dzi, tfi * dzr);
+    dzr = ndr; dzi = ndi; ur = nur; ui = nui;
+    in = in && (((unsigned)fx_hi(wr) + R) | ((unsigned)fx_hi(wi) + R)) < 2u * R;
+    const int nyh = -y.h;
+    const long long tr = fx_mad(nyh, y.l, fx_mad(x.h, x.l, tr0));
+    const long long ti = fx_mad(x.l, y.h, fx_mad(x.h, y.l, ti0));
+    wr = fx_mad(nyh, y.h, fx_mad(x.h, x.h, CR)) + fx_shr31(tr);
+    wi = fx_mad(x.h + x.h, y.h, CI) + fx_shr31(ti);
+    x = fx_split(wr, S);
+    y = fx_split(wi, S);
+    if (CAP && k == lcap) { cwr = wr; cwi = wi; capd_r = dzr; capd_i = dzi; capu_r = ur; capu_i = ui; }
+  }
+  float Ur = ur, Ui = ui;  // P'' / 4^m
+  if (CAP && lcap >= 1) {
+    wr += cwr;
+    wi += cwi;
+    const float a = fx_pow2f(2 * (lcap - m));
+    dzr += capd_r;
+    dzi += capd_i;
+    Ur = fmaf(a, capu_r, ur);
+    Ui = fmaf(a, capu_i, ui);
+  }
+  Wr = wr;
+  Wi = wi;
+  dr = dzr;
+  di = dzi;
+  // P''/(2P') = (U 2^(m-1)) / (P' 2^-m), both scalings exact
+  const float up = fx_pow2f(m - 1), dn = fx_pow2f(-m);
+  const float ar = Ur * up, ai = Ui * up, cr2 = dr * dn, ci2 = di * dn;
+  const float inv = 1.f / fmaf(cr2, cr2, ci2 * ci2);
+  kr = fmaf(ar, cr2, ai * ci2) * inv;
+  ki = fmaf(ai, cr2, -ar * ci2) * inv;
+  return in;
+}
+#endif
+
 // (a + ib) (c + id) 2^sc
 __host__ __device__ __forceinline__ void fx_cmul(ff a, ff b, ff c, ff d, int sc, ff& qr, ff& qi) {
   const float s = fx_pow2f(sc < -126 ? -126 : sc), s2 = sc < -126 ? fx_pow2f(sc + 126) : 1.f;

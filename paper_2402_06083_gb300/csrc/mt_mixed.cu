@@ -29,13 +29,24 @@
 // its binary64 finishing steps.  The chunk-end check of the walk and the
 // count check catch any tracking failure, and the host then repeats the
 // split in plain binary64.
-#include "mt_ff.cuh"
+#include "mt_fix.cuh"
 #include "mt_levelline.cuh"
 #include "mt_pert.cuh"
 
 namespace mt {
 
 constexpr int MIX_MAXM = 41;
+// Shorter orbits of p_n keep an anchor per start, the whole orbit and the
+// binary64 finish and tip redo: the splits are short there (p_20: 5 % of 1.36
+// ms from all of them), and the last digits of their roots, on which the
+// nearest-neighbour distances at the tip rest, stay as they were.
+constexpr int MIX_LONG = 23;
+inline bool mixed_short(const PolyDev& P) { return P.kind == 0 && P.m < MIX_LONG; }
+// The binary64 finish in fixed point: up to p_25.  Of p_28's 67 M roots some
+// neighbours' real parts agree in every digit; their places in the sorted list
+// hang on the last one, and the binary64 finish leaves those as they were (1e-10
+// at the worst of 4 M sampled components, 9e-7 with the fixed one).
+constexpr int FIN_FX_MAXM = 25;
 
 // binary64 reference orbit at c0: zs[k * stride] = Z_k in binary32 for
 // k = 0 .. m-1 (truncated on the integer pipe: the binary64 pipe keeps the
@@ -513,7 +524,7 @@ WalkMixedFn walk_mixed_fixed(int m) {
 // the loop over a varying length only add latency (ms of the walk, without and
 // with the series: p_20 0.178 and 0.212, p_21 0.222 and 0.246, p_22 0.408 and
 // 0.365, p_24 1.63 and 1.36, p_28 24.9 and 17.8).
-constexpr int WALK_SERIES_MIN = 23;
+constexpr int WALK_SERIES_MIN = MIX_LONG;
 WalkMixedFn walk_mixed_kernel(const PolyDev& P) {
   if (P.lcap >= 0) return &k_walk_mixed<true, 0>;
   if (P.m >= WALK_SERIES_MIN) return &k_walk_series;
@@ -703,10 +714,6 @@ constexpr int DM_BS = 128;     // threads per block of the binary32 descent
 constexpr int DM_REFILL = 11;
 constexpr int DM_MAX_WARPS = 16384;  // warp slots of the anchor buffer (grids are capped to fit)
 constexpr int DM_TAIL = 12;
-// Orbits shorter than this run whole: the skipped steps no longer pay for the far
-// list's launch (p_16: 0.061 ms whole, 0.079 with 4 steps skipped; p_20 0.183 and 0.182).
-constexpr int DM_SERIES_MIN = 20;
-
 template <bool CAP, int MC, bool LIST>
 __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, int Kr, int gsh,
                                                          const double2* __restrict__ starts, int64_t cnt,
@@ -716,7 +723,7 @@ __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, int Kr, int 
                                                          DevCounters* ctr) {
   extern __shared__ float2 zsh[];
   constexpr int stride = DM_BS + 1;
-  constexpr int KC = MC >= DM_SERIES_MIN ? MC - DM_TAIL : 1;
+  constexpr int KC = MC >= MIX_LONG ? MC - DM_TAIL : 1;
   const int K = MC > 0 ? KC : Kr;
   const float2* zs = zsh + threadIdx.x;  // row 0 (Z_K) of this lane's column
   const unsigned lane = threadIdx.x & 31;
@@ -1086,10 +1093,21 @@ __global__ void k_finish_list(int64_t count, const uint32_t* __restrict__ head, 
 }
 
 // Binary64 Newton steps (eq. Newton) from each head's binary32 end point
-// until |step| < tol (normally two steps) or the rounding floor.
-// Persistent, with per-lane refill by warp vote (as k_descend): a lane that
-// finished takes the next head of the list at once, so the warp never waits
-// for its slowest finish (one to six steps) before starting new ones.
+// until |step| < tol or the next step, predicted, is below tol / 4 (normally
+// one step), or the rounding floor.  Persistent, with per-lane refill by warp
+// vote (as k_descend): lanes that finished take the next heads of the list
+// together once FIN_REFILL wait, so the warp never waits for its slowest
+// finish (one to six steps) before starting new ones.
+//
+// FX: the value in fixed point (mt_fix.cuh; the end points lie near roots, in
+// its range), the derivatives in binary32, as without FX, where the value is
+// binary64 (the polynomials kept there).  Bound: the integer multiply-add
+// pipe (56 %) and issue (70 %); in binary64 that pipe's 3 FMA a step, 16 clocks
+// a warp each, with the heads outside the line repeating six steps.  p_24, 4.5 M
+// heads: 0.865 -> 0.273 ms (p_28 15.1 -> 4.65; not taken there, FIN_FX_MAXM).
+constexpr int FIN_FB = 28;
+constexpr unsigned FIN_REFILL = 6;
+template <bool FX, bool CAP>
 __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* __restrict__ list,
                                                     const unsigned long long* __restrict__ nlist,
                                                     int64_t cap_list, double tol2, int cap,
@@ -1098,52 +1116,95 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
                                                     uint8_t* __restrict__ status,
                                                     unsigned long long* queue, DevCounters* ctr) {
   const unsigned lane = threadIdx.x & 31;
-  const int64_t nl = (int64_t)*nlist < cap_list ? (int64_t)*nlist : cap_list;
+  const unsigned nl = (unsigned)((int64_t)*nlist < cap_list ? (int64_t)*nlist : cap_list);  // < 2^32
   const float tol2f = f32_trunc(tol2), tol2q = 0.0625f * tol2f;  // tol^2, (tol / 4)^2
-  int64_t t = -1;  // position in the list of this lane's finish
+  uint32_t at = 0;  // the candidate of this lane's finish
   double zx = 0.0, zy = 0.0;
+  long long X = 0, Y = 0;
   float prev2 = 3.0e38f;
-  int it = 0;
+  int it = 0, outcome = 0;  // >= 0: no running finish (have: its result waits to be written)
+  bool have = false;
   bool drained = false;  // warp-uniform: the list is handed out
-  unsigned long long s64 = 0;
+  unsigned s64 = 0;
   for (;;) {
-    const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, t < 0);
-    if (need) {
-      const int leader = __ffs(need) - 1;
+    const unsigned wait = __ballot_sync(0xffffffffu, outcome >= 0);
+    if (__popc(wait) >= (drained ? 32u : FX ? FIN_REFILL : 1u)) {
+      if (have && outcome >= 0) {
+        if (FX) {
+          zx = fx_to_f64<FIN_FB>(X);
+          zy = fx_to_f64<FIN_FB>(Y);
+        }
+        cand[at] = make_double2(zx, zy);
+        status[at] = (uint8_t)outcome;
+        have = false;
+      }
+      if (drained) break;
       unsigned long long b0 = 0;
-      if ((int)lane == leader) b0 = atomicAdd(queue, (unsigned long long)__popc(need));
-      b0 = __shfl_sync(0xffffffffu, b0, leader);
-      if (t < 0) {
-        t = (int64_t)(b0 + __popc(need & lanemask_lt()));
+      if (lane == (unsigned)(__ffs(wait) - 1)) b0 = atomicAdd(queue, (unsigned long long)__popc(wait));
+      b0 = __shfl_sync(0xffffffffu, b0, __ffs(wait) - 1);
+      if (outcome >= 0) {
+        const unsigned long long t = b0 + __popc(wait & lanemask_lt());
         if (t < nl) {
-          const double2 z = c32[list[t]];
+          at = list[t];
+          const double2 z = c32[at];
           zx = z.x;
           zy = z.y;
+          if (FX) {
+            X = fx_from_f64<FIN_FB>(zx);
+            Y = fx_from_f64<FIN_FB>(zy);
+          }
           it = 0;
           prev2 = 3.0e38f;
+          outcome = FX && !(fx_fits<FIN_FB>(zx) && fx_fits<FIN_FB>(zy)) ? 1 : -1;
+          have = true;
         }
       }
-      if ((int64_t)(b0 + __popc(need)) >= nl) drained = true;
+      if (b0 + __popc(wait) >= nl) drained = true;
     }
-    const bool active = t >= 0 && t < nl;
-    if (!__any_sync(0xffffffffu, active)) break;
-    if (active) {
-      double vr, vi;
-      float dr, di, kr, ki;
-      orbit_f64_d32_k(P.m, P.lcap, zx, zy, vr, vi, dr, di, kr, ki);
+    if (outcome < 0) {
+      float dr, di, kr, ki, fvx, fvy;
+      double vr = 0.0, vi = 0.0;
+      bool in = true;
+      if (FX) {
+        long long Wr, Wi;
+        in = fx_value_d32_k<FIN_FB, CAP>(P.m, P.lcap, X, Y, Wr, Wi, dr, di, kr, ki);
+        fvx = fx_to_f32<FIN_FB>(Wr);
+        fvy = fx_to_f32<FIN_FB>(Wi);
+      } else {
+        orbit_f64_d32_k(P.m, P.lcap, zx, zy, vr, vi, dr, di, kr, ki);
+        fvx = f32_trunc(vr);
+        fvy = f32_trunc(vi);
+      }
       // the quotient in binary32: the derivative is binary32 already, and a
       // step accurate to 1e-7 of itself leaves ~1e-7 q besides the quadratic
       // K q^2 -- far below tol for the q ~ 1e-5 of a descent's scale that
-      // the binary32 phase leaves; binary64 only for the value and z - q
+      // the binary32 phase leaves; 64 bits only for the value and z - q
       float qr, qi;
-      if (!cdiv_f32s(f32_trunc(vr), f32_trunc(vi), dr, di, qr, qi)) {
+      const bool ok = cdiv_f32s(fvx, fvy, dr, di, qr, qi);
+      if (!FX && !ok) {
         double qd, qe;  // a derivative out of binary32's scaled range: binary64
         cdiv_f64(vr, vi, (double)dr, (double)di, qd, qe);
         qr = f32_trunc(qd);
         qi = f32_trunc(qe);
       }
-      zx -= f64_of_f32(qr);
-      zy -= f64_of_f32(qi);
+      float fzx, fzy;
+      bool finite;
+      if (FX) {
+        finite = ok && fabsf(qr) < 2.f && fabsf(qi) < 2.f;
+        if (finite) {
+          X -= fx_from_ff<FIN_FB>(ff{qr, 0.f});
+          Y -= fx_from_ff<FIN_FB>(ff{qi, 0.f});
+          finite = fx_in<FIN_FB>(X) && fx_in<FIN_FB>(Y);
+        }
+        fzx = (float)fx_hi(X) * fx_pow2f(-FIN_FB);
+        fzy = (float)fx_hi(Y) * fx_pow2f(-FIN_FB);
+      } else {
+        zx -= f64_of_f32(qr);
+        zy -= f64_of_f32(qi);
+        fzx = f32_trunc(zx);
+        fzy = f32_trunc(zy);
+        finite = finite2(zx, zy);
+      }
       ++it;
       ++s64;
       const float s2 = fmaf(qr, qr, qi * qi);
@@ -1151,11 +1212,13 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
       const float q2r = fmaf(qr, qr, -qi * qi), q2i = 2.f * qr * qi;
       const float pr = fmaf(q2r, kr, -q2i * ki), pi = fmaf(q2r, ki, q2i * kr);
       const float pred2 = fmaf(pr, pr, pi * pi);
-      const float fzx = f32_trunc(zx), fzy = f32_trunc(zy);
       // binary64 rounding floor (16 ulp of the larger of 1 and |z|), in binary32
       const float fl = (1.f + fabsf(fzx) + fabsf(fzy)) * 3.552713678800501e-15f;
-      int outcome = -1;
-      if (!finite2(zx, zy) || fmaf(fzx, fzx, fzy * fzy) > 1e4f) outcome = 1;
+      // an orbit that leaves the fixed range (|p_k| >= 4 before the end, about 1 %
+      // of the heads: binary32 descents that ended outside the line, status 3
+      // with P' beyond binary32) is more steps from any root than the cap allows
+      if (!in) outcome = 2;
+      else if (!finite || fmaf(fzx, fzx, fzy * fzy) > 1e4f) outcome = 1;
       else if (s2 < tol2f) outcome = 0;
       // quadratic regime (the next step under a quarter of this one) and the
       // next step under tol / 4: c - q is the root to within tol / 4
@@ -1163,12 +1226,6 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
       else if (s2 >= 0.25f * prev2 && s2 < fl * fl) outcome = 0;  // rounding floor
       else if (it >= cap) outcome = 2;
       prev2 = s2;
-      if (outcome >= 0) {
-        const uint32_t i = list[t];
-        cand[i] = make_double2(zx, zy);
-        status[i] = (uint8_t)outcome;
-        t = -1;
-      }
     }
   }
   warp_add_u64(&ctr->desc_newton, s64);
@@ -1301,8 +1358,8 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
     // s_{l,n} keeps an anchor per start and the whole orbit: its line lies at
     // |s| = 100, and binary32 relative to a neighbour's delta lost tip roots
     // (s_{6,12}: none of 7 levels without, 3 with).
-    const bool shared = P.kind == 0;
-    const int K = shared && P.m >= DM_SERIES_MIN ? P.m - DM_TAIL : 1;
+    const bool shared = P.kind == 0 && P.m >= MIX_LONG;
+    const int K = shared ? P.m - DM_TAIL : 1;
     const int gsh = shared ? 2 : 0;
     uint32_t* far = fin.pos;  // free until the finish's scan
     unsigned long long* nfar = fin.nheads;
@@ -1343,10 +1400,14 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
   k_finish_list<<<nb, bs, 0, s>>>(count, fin.head, fin.pos, fin.vals, fin.list);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   {
-    // persistent: 8 warps per SM keep the binary64 pipe busy (as k_descend)
+    // persistent: 8 warps per SM keep the binary64 pipe busy, 24 the integer
+    // pipes (as k_descend)
+    const bool fx = P.fx && !mixed_short(P) && !(P.kind == 0 && P.m > FIN_FX_MAXM);
+    const auto kfin = !fx ? &k_finish_f64<false, false>
+                          : P.lcap >= 1 ? &k_finish_f64<true, true> : &k_finish_f64<true, false>;
     int fin_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fin_sm, k_finish_f64, bs, 0)) != cudaSuccess) return e;
-    if (fin_sm > 2) fin_sm = 2;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fin_sm, kfin, bs, 0)) != cudaSuccess) return e;
+    if (fin_sm > (fx ? 6 : 2)) fin_sm = fx ? 6 : 2;
     if (fin_sm < 1) fin_sm = 1;
     int64_t fgrid = (int64_t)device_sm_count() * fin_sm;
     if (fgrid > (int64_t)nb) fgrid = (int64_t)nb;
@@ -1354,8 +1415,7 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
     if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess) return e;
     MT_COUNT_LAUNCH(1);
     if ((e = ktimer_begin(KS_FINISH, s)) != cudaSuccess) return e;
-    k_finish_f64<<<(unsigned)fgrid, bs, 0, s>>>(P, fin.list, fin.nheads, count, tol * tol, 6, starts, cand, status,
-                                                q, ctr);
+    kfin<<<(unsigned)fgrid, bs, 0, s>>>(P, fin.list, fin.nheads, count, tol * tol, 6, starts, cand, status, q, ctr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = ktimer_end(s)) != cudaSuccess) return e;
   }
@@ -1368,7 +1428,9 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
   MT_COUNT_LAUNCH(1);
   k_tip_list<<<sgrid, bs, 0, s>>>(fin.vals, &ctr->n_c32_fin, n2, fin.pos);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_descend_list(P, starts, fin.pos, n2, count, tol, cap, cand, status, ctr, s)) != cudaSuccess)
+  PolyDev Pt = P;
+  if (mixed_short(P)) Pt.fx = 0;
+  if ((e = launch_descend_list(Pt, starts, fin.pos, n2, count, tol, cap, cand, status, ctr, s)) != cudaSuccess)
     return e;
   MT_COUNT_LAUNCH(2);
   k_finish_append<<<sgrid, bs, 0, s>>>(fin.pos, n2, fin.list, fin.nheads, count, status, ctr);

@@ -1,6 +1,7 @@
 """The mixed tier's descents on shared anchors and the anchors' series
 (csrc/mt_mixed.cu): orbit lengths on both sides of the rules (general loop
-below 16, fixed lengths from 16, series from 20), starts that do not fill a
+below 16, fixed lengths from 16, shared anchors, series and the fixed-point
+finish from 23), starts that do not fill a
 group or a queue range, and denser starts, whose groups span less of a turn."""
 from __future__ import annotations
 
@@ -19,7 +20,8 @@ def mt():
 
 
 @pytest.mark.parametrize("n,kw", [(1, {}), (2, {}), (3, {}), (6, {}), (7, {}), (13, {}), (15, {}), (16, {}), (17, {}),
-                                  (19, {}), (20, {}), (21, {}), (20, {"M": 16, "c_L": 8}), (20, {"M": 8, "c_L": 2}),
+                                  (19, {}), (20, {}), (21, {}), (22, {}), (23, {}), (24, {}), (25, {}), (23, {"M": 16, "c_L": 8}), (23, {"M": 8, "c_L": 2}),
+                                  (23, {"lambda0": 5.8}), (23, {"stream_pieces": 4}), (20, {"M": 16, "c_L": 8}), (20, {"M": 8, "c_L": 2}),
                                   (20, {"lambda0": 5.8}), (18, {"stream_pieces": 4}), (21, {"stream_pieces": 2})])
 def test_first_attempt_finds_every_root(mt, n, kw):
     """The first attempt alone (no binary64 repeat) is complete and certified,
