@@ -406,8 +406,8 @@ __device__ __forceinline__ float fx_to_f32(long long w) {
 // 2^-2FB, P' and the curvature P'' / (2 P') in binary32.  False where the
 // orbit leaves the fixed range before its last step.  The value alone is a
 // third of fx_eval's step; its binary32 companions run beside it.
-template <int FB, bool CAP>
-__device__ __forceinline__ bool fx_value_d32_k(int m, int lcap, long long X, long long Y, long long& Wr, long long& Wi,
+template <int FB>
+__device__ __forceinline__ bool fx_value_d32_k(int m, long long X, long long Y, long long& Wr, long long& Wi,
                                                float& dr, float& di, float& kr, float& ki) {
   constexpr int S = 32 - FB;
   constexpr unsigned R = 1u << (FB - 2);
@@ -415,10 +415,9 @@ __device__ __forceinline__ bool fx_value_d32_k(int m, int lcap, long long X, lon
   const long long tr0 = ((X - (CR << S)) << (31 - S)) + (1ll << 30);
   const long long ti0 = ((Y - (CI << S)) << (31 - S)) + (1ll << 30);
   fx2 x = fx_split(X, 0), y = fx_split(Y, 0);
-  long long wr = CR, wi = CI, cwr = 0, cwi = 0;
-  float dzr = 1.f, dzi = 0.f, capd_r = 0.f, capd_i = 0.f;  // p'_1 = 1, p''_1 = 0
-  float ur = 0.f, ui = 0.f, capu_r = 0.f, capu_i = 0.f;
-  if (CAP && lcap == 1) { cwr = wr; cwi = wi; capd_r = 1.f; }
+  long long wr = CR, wi = CI;
+  float dzr = 1.f, dzi = 0.f;  // p'_1 = 1, p''_1 = 0
+  float ur = 0.f, ui = 0.f;  // p''_k / 4^k
   float h = 0.5f;  // 2^-(k-1), k = 2
   bool in = true;
 #pragma unroll 4
@@ -440,25 +439,14 @@ __device__ __forceinline__ bool fx_value_d32_k(int m, int lcap, long long X, lon
     wi = fx_mad(x.h + x.h, y.h, CI) + fx_shr31(ti);
     x = fx_split(wr, S);
     y = fx_split(wi, S);
-    if (CAP && k == lcap) { cwr = wr; cwi = wi; capd_r = dzr; capd_i = dzi; capu_r = ur; capu_i = ui; }
-  }
-  float Ur = ur, Ui = ui;  // P'' / 4^m
-  if (CAP && lcap >= 1) {
-    wr += cwr;
-    wi += cwi;
-    const float a = fx_pow2f(2 * (lcap - m));
-    dzr += capd_r;
-    dzi += capd_i;
-    Ur = fmaf(a, capu_r, ur);
-    Ui = fmaf(a, capu_i, ui);
   }
   Wr = wr;
   Wi = wi;
   dr = dzr;
   di = dzi;
-  // P''/(2P') = (U 2^(m-1)) / (P' 2^-m), both scalings exact
+  // P''/(2P') = (u 2^(m-1)) / (P' 2^-m), both scalings exact
   const float up = fx_pow2f(m - 1), dn = fx_pow2f(-m);
-  const float ar = Ur * up, ai = Ui * up, cr2 = dr * dn, ci2 = di * dn;
+  const float ar = ur * up, ai = ui * up, cr2 = dr * dn, ci2 = di * dn;
   const float inv = 1.f / fmaf(cr2, cr2, ci2 * ci2);
   kr = fmaf(ar, cr2, ai * ci2) * inv;
   ki = fmaf(ai, cr2, -ar * ci2) * inv;

@@ -42,10 +42,12 @@ constexpr int MIX_MAXM = 41;
 // nearest-neighbour distances at the tip rest, stay as they were.
 constexpr int MIX_LONG = 23;
 inline bool mixed_short(const PolyDev& P) { return P.kind == 0 && P.m < MIX_LONG; }
-// The binary64 finish in fixed point: up to p_25.  Of p_28's 67 M roots some
+// The binary64 finish in fixed point: p_23 to p_25.  Of p_28's 67 M roots some
 // neighbours' real parts agree in every digit; their places in the sorted list
 // hang on the last one, and the binary64 finish leaves those as they were (1e-10
-// at the worst of 4 M sampled components, 9e-7 with the fixed one).
+// at the worst of 4 M sampled components, 9e-7 with the fixed one).  s_{l,n}
+// keeps it too: at |s| = 100 its tip pairs rest on the same digits (q_{8,12}: 4411
+// roots to redo in double-double with the fixed finish, over the 4096 places).
 constexpr int FIN_FX_MAXM = 25;
 
 // binary64 reference orbit at c0: zs[k * stride] = Z_k in binary32 for
@@ -1107,7 +1109,7 @@ __global__ void k_finish_list(int64_t count, const uint32_t* __restrict__ head, 
 // heads: 0.865 -> 0.273 ms (p_28 15.1 -> 4.65; not taken there, FIN_FX_MAXM).
 constexpr int FIN_FB = 28;
 constexpr unsigned FIN_REFILL = 6;
-template <bool FX, bool CAP>
+template <bool FX>
 __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* __restrict__ list,
                                                     const unsigned long long* __restrict__ nlist,
                                                     int64_t cap_list, double tol2, int cap,
@@ -1167,7 +1169,7 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
       bool in = true;
       if (FX) {
         long long Wr, Wi;
-        in = fx_value_d32_k<FIN_FB, CAP>(P.m, P.lcap, X, Y, Wr, Wi, dr, di, kr, ki);
+        in = fx_value_d32_k<FIN_FB>(P.m, X, Y, Wr, Wi, dr, di, kr, ki);
         fvx = fx_to_f32<FIN_FB>(Wr);
         fvy = fx_to_f32<FIN_FB>(Wi);
       } else {
@@ -1402,9 +1404,8 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
   {
     // persistent: 8 warps per SM keep the binary64 pipe busy, 24 the integer
     // pipes (as k_descend)
-    const bool fx = P.fx && !mixed_short(P) && !(P.kind == 0 && P.m > FIN_FX_MAXM);
-    const auto kfin = !fx ? &k_finish_f64<false, false>
-                          : P.lcap >= 1 ? &k_finish_f64<true, true> : &k_finish_f64<true, false>;
+    const bool fx = P.fx && P.kind == 0 && !mixed_short(P) && P.m <= FIN_FX_MAXM;
+    const auto kfin = fx ? &k_finish_f64<true> : &k_finish_f64<false>;
     int fin_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fin_sm, kfin, bs, 0)) != cudaSuccess) return e;
     if (fin_sm > (fx ? 6 : 2)) fin_sm = fx ? 6 : 2;
