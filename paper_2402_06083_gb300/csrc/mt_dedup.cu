@@ -11,6 +11,8 @@
 // the earlier candidates of its Re window -> exclusive scan -> gather.
 // Every kernel is a coalesced pass over HBM; the radix sort ranks keys
 // stably inside a block (digit peers of a warp by ballots).
+#include <cooperative_groups.h>
+
 #include "mt_common.cuh"
 
 namespace mt {
@@ -177,34 +179,31 @@ __global__ void k_scan_sums(unsigned long long* sums, int64_t nb, unsigned long 
   if (threadIdx.x == 0 && total) *total = tot;
 }
 
-__global__ void k_scan_tiles(const uint32_t* in, uint32_t* out, int64_t n,
-                             const unsigned long long* __restrict__ sums) {
-  __shared__ unsigned long long sh[32];
-  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-  // each thread owns SCAN_ITEMS consecutive elements (blocked arrangement)
-  const int64_t t0 = base + (int64_t)threadIdx.x * SCAN_ITEMS;
-  // a full run of 8 moves as two 16-byte words where both buffers are
-  // 16-byte aligned (t0 is a multiple of 8)
-  const bool full = t0 + SCAN_ITEMS <= n && ((((uintptr_t)in) | ((uintptr_t)out)) & 15u) == 0;
-  uint32_t v[SCAN_ITEMS];
-  unsigned long long acc = 0;
-  if (full) {
+// A thread's run of SCAN_ITEMS elements from t0 on (blocked arrangement; 0
+// beyond n).  A full run of 8 moves as two 16-byte words where both buffers are
+// 16-byte aligned (t0 is a multiple of 8).
+__device__ __forceinline__ bool scan_wide(const uint32_t* in, const uint32_t* out, int64_t t0, int64_t n) {
+  return t0 + SCAN_ITEMS <= n && ((((uintptr_t)in) | ((uintptr_t)out)) & 15u) == 0;
+}
+__device__ __forceinline__ void scan_load(const uint32_t* in, const uint32_t* out, int64_t t0, int64_t n,
+                                          uint32_t (&v)[SCAN_ITEMS]) {
+  if (scan_wide(in, out, t0, n)) {
     const uint4 a = *(const uint4*)(in + t0), b = *(const uint4*)(in + t0 + 4);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   } else {
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = (t0 + k < n) ? in[t0 + k] : 0u;
   }
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) acc += v[k];
-  unsigned long long off = block_excl_scan_u64(acc, sh, nullptr) + sums[blockIdx.x];
+}
+__device__ __forceinline__ void scan_store(const uint32_t* in, uint32_t* out, int64_t t0, int64_t n,
+                                           const uint32_t (&v)[SCAN_ITEMS], unsigned long long off) {
   uint32_t o[SCAN_ITEMS];
 #pragma unroll
   for (int k = 0; k < SCAN_ITEMS; ++k) {
     o[k] = (uint32_t)off;
     off += v[k];
   }
-  if (full) {
+  if (scan_wide(in, out, t0, n)) {
     *(uint4*)(out + t0) = make_uint4(o[0], o[1], o[2], o[3]);
     *(uint4*)(out + t0 + 4) = make_uint4(o[4], o[5], o[6], o[7]);
   } else {
@@ -212,6 +211,44 @@ __global__ void k_scan_tiles(const uint32_t* in, uint32_t* out, int64_t n,
     for (int k = 0; k < SCAN_ITEMS; ++k)
       if (t0 + k < n) out[t0 + k] = o[k];
   }
+}
+
+__global__ void k_scan_tiles(const uint32_t* in, uint32_t* out, int64_t n,
+                             const unsigned long long* __restrict__ sums) {
+  __shared__ unsigned long long sh[32];
+  const int64_t t0 = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
+  uint32_t v[SCAN_ITEMS];
+  scan_load(in, out, t0, n, v);
+  unsigned long long acc = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_ITEMS; ++k) acc += v[k];
+  const unsigned long long off = block_excl_scan_u64(acc, sh, nullptr) + sums[blockIdx.x];
+  scan_store(in, out, t0, n, v, off);
+}
+
+// Short scans in one launch: one block takes SCAN_ONE_TILE elements a round and
+// carries the sum.  Bound: launches (the three of the general scan take about
+// 4 us each, whatever the size).  8192 elements: 12.0 -> 5.6 us, 16385 13.1 ->
+// 10.0, 32768 13.5 -> 11.7; beyond, the one block is the slower.
+constexpr int SCAN_ONE_BS = 1024;
+constexpr int64_t SCAN_ONE_TILE = (int64_t)SCAN_ONE_BS * SCAN_ITEMS;
+constexpr int64_t SCAN_ONE_MAX = 4 * SCAN_ONE_TILE;
+__global__ void __launch_bounds__(SCAN_ONE_BS) k_scan_one(const uint32_t* in, uint32_t* out, int64_t n,
+                                                          unsigned long long* total) {
+  __shared__ unsigned long long sh[32];
+  unsigned long long carry = 0;
+  for (int64_t base = 0; base < n; base += SCAN_ONE_TILE) {
+    const int64_t t0 = base + (int64_t)threadIdx.x * SCAN_ITEMS;
+    uint32_t v[SCAN_ITEMS];
+    scan_load(in, out, t0, n, v);
+    unsigned long long acc = 0, tot;
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) acc += v[k];
+    const unsigned long long off = block_excl_scan_u64(acc, sh, &tot) + carry;
+    carry += tot;
+    scan_store(in, out, t0, n, v, off);
+  }
+  if (threadIdx.x == 0 && total) *total = carry;
 }
 
 size_t scan_temp_bytes(int64_t n) {
@@ -222,6 +259,11 @@ size_t scan_temp_bytes(int64_t n) {
 cudaError_t launch_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, void* temp,
                                   unsigned long long* total, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
+  if (n <= SCAN_ONE_MAX) {
+    MT_COUNT_LAUNCH(1);
+    k_scan_one<<<1, SCAN_ONE_BS, 0, s>>>(in, out, n, total);
+    return cudaGetLastError();
+  }
   const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
   unsigned long long* sums = (unsigned long long*)temp;
   MT_COUNT_LAUNCH(1);
@@ -483,6 +525,160 @@ size_t radix_temp_bytes(int64_t n) {
   return (size_t)nh * 2 * sizeof(uint32_t) + 256 * sizeof(uint32_t);
 }
 
+// Small sorts: every pass in one launch of one thread-block cluster.
+//
+// Up to RC_MAX elements the three launches of a pass are latency, not traffic
+// (24 launches for a root set, about 5 us each).  Here each of RC_BLOCKS blocks
+// owns a contiguous run of positions in its shared memory; a pass ranks the
+// run in registers as k_rs_scatter does, reads the blocks' digit counts from
+// their shared memory, and writes each element to its new owner's (distributed
+// shared memory): two cluster barriers a pass, and global memory only before
+// the first pass and in the last.  The order is the stable one, the same as
+// that of the pass-wise sort.
+//
+// Bound: the two barriers and the chain of a pass (ranks, prefix over the
+// warps, remote counts, digit scan).  Root sets (8 passes): 4097 elements
+// 117 -> 33 us, 16385 141 -> 60, 40960 143 -> 90, where a block's registers and
+// shared memory end; finish keys (5 passes): 4097 83 -> 24, 40960 83 -> 60.
+constexpr int RC_BLOCKS = 8;  // the portable cluster size
+constexpr int RC_BS = 1024;
+constexpr int RC_WARPS = RC_BS / 32;
+constexpr int RC_ITEMS = 5;  // 2^15 starts and one are 4097 a block
+constexpr int RC_RUN = RC_BS * RC_ITEMS;
+constexpr int64_t RC_MAX = (int64_t)RC_BLOCKS * RC_RUN;
+constexpr int RC_ROW = 257;  // the quarter prefixes of a digit fall on different banks
+constexpr size_t RC_SMEM = RC_RUN * (sizeof(uint64_t) + sizeof(uint32_t)) + RC_WARPS * RC_ROW * sizeof(uint32_t);
+
+__global__ void __cluster_dims__(RC_BLOCKS, 1, 1) __launch_bounds__(RC_BS)
+    k_rs_cluster(uint64_t* keys, uint32_t* vals, int64_t cap, int begin_bit, int end_bit,
+                 const unsigned long long* __restrict__ n_dev) {
+  extern __shared__ uint64_t rc_smem[];
+  uint64_t* sk = rc_smem;
+  uint32_t* sv = (uint32_t*)(sk + RC_RUN);
+  uint32_t* wc = sv + RC_RUN;      // [warp][digit]: running count, then the warps-before prefix
+  __shared__ uint32_t gpos[256];   // position of the block's first element of digit d
+  __shared__ uint32_t cnt[256];    // this block's digit counts, read by the cluster
+  __shared__ uint32_t wsum[8];
+  const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const unsigned me = cl.block_rank();
+  const unsigned n = (unsigned)rs_count(cap, n_dev);
+  // items a lane, and elements a warp and a block hold
+  const unsigned ni = (n + RC_BLOCKS * RC_BS - 1) / (RC_BLOCKS * RC_BS);
+  const unsigned run = RC_BS * ni;
+  const unsigned l0 = w * (32 * ni) + lane;  // the thread's first element of the block's run
+  const unsigned g0 = me * run + l0;
+  uint64_t key[RC_ITEMS];
+  uint32_t val[RC_ITEMS];
+#pragma unroll
+  for (int k = 0; k < RC_ITEMS; ++k) {
+    const bool valid = k < ni && g0 + k * 32 < n;
+    key[k] = valid ? keys[g0 + k * 32] : 0ull;
+    val[k] = valid ? vals[g0 + k * 32] : 0u;
+  }
+  // no block writes keys or vals before every block has loaded its run: the
+  // last pass writes them after the first pass's barrier
+  uint32_t* row = wc + w * RC_ROW;
+  for (int shift = begin_bit; shift < end_bit; shift += 8) {
+#pragma unroll
+    for (int q = 0; q < 256 / 32; ++q) row[lane + 32 * q] = 0;
+    __syncwarp();
+    unsigned dg[RC_ITEMS], rk[RC_ITEMS];
+#pragma unroll
+    for (int k = 0; k < RC_ITEMS; ++k) {
+      if (k >= ni) break;
+      const bool valid = g0 + k * 32 < n;
+      dg[k] = valid ? (unsigned)(key[k] >> shift) & 255u : 256u;
+      const unsigned peers = rs_peers<true>(dg[k]);
+      const unsigned lt = __popc(peers & lanemask_lt());
+      const uint32_t before = valid ? row[dg[k]] : 0u;
+      __syncwarp();
+      if (valid && lt == 0) row[dg[k]] = before + __popc(peers);
+      __syncwarp();
+      rk[k] = before + lt;
+    }
+    __syncthreads();
+    {  // prefix over the warps: four threads a digit, eight warps each
+      const int d = t >> 2, part = t & 3;
+      uint32_t c[RC_WARPS / 4], r = 0;
+#pragma unroll
+      for (int q = 0; q < RC_WARPS / 4; ++q) c[q] = wc[(part * (RC_WARPS / 4) + q) * RC_ROW + d];
+#pragma unroll
+      for (int q = 0; q < RC_WARPS / 4; ++q) r += c[q];
+      uint32_t x = r;
+      for (int o = 1; o < 4; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o, 4);
+        if (part >= o) x += y;
+      }
+      if (part == 3) cnt[d] = x;
+      x -= r;
+#pragma unroll
+      for (int q = 0; q < RC_WARPS / 4; ++q) {
+        wc[(part * (RC_WARPS / 4) + q) * RC_ROW + d] = x;
+        x += c[q];
+      }
+    }
+    cl.sync();  // the counts are out, and every run is in registers
+    uint32_t before = 0, total = 0, x = 0;
+    if (t < 256) {
+      uint32_t c[RC_BLOCKS];
+#pragma unroll
+      for (int b = 0; b < RC_BLOCKS; ++b) c[b] = cl.map_shared_rank(cnt, b)[t];
+#pragma unroll
+      for (int b = 0; b < RC_BLOCKS; ++b) {
+        if (b < (int)me) before += c[b];
+        total += c[b];
+      }
+      x = total;  // exclusive scan over the digits
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) wsum[w] = x;
+    }
+    __syncthreads();
+    if (t < 256) {
+      for (int q = 0; q < 8; ++q) before += q < w ? wsum[q] : 0u;
+      gpos[t] = before + x - total;
+    }
+    __syncthreads();
+    const bool last = shift + 8 >= end_bit;
+#pragma unroll
+    for (int k = 0; k < RC_ITEMS; ++k) {
+      if (k >= ni) break;
+      if (dg[k] >= 256u) continue;
+      const unsigned pos = gpos[dg[k]] + row[dg[k]] + rk[k];
+      if (last) {
+        keys[pos] = key[k];
+        vals[pos] = val[k];
+      } else {
+        const unsigned b = pos / run, p = pos - b * run;
+        cl.map_shared_rank(sk, b)[p] = key[k];
+        cl.map_shared_rank(sv, b)[p] = val[k];
+      }
+    }
+    // the runs are complete, the counts may be overwritten, and after the last
+    // pass the block may leave
+    cl.sync();
+    if (last) break;
+#pragma unroll
+    for (int k = 0; k < RC_ITEMS; ++k) {
+      if (k >= ni) break;
+      key[k] = sk[l0 + k * 32];
+      val[k] = sv[l0 + k * 32];
+    }
+  }
+}
+
+static cudaError_t rs_cluster(uint64_t* keys, uint32_t* vals, int64_t n, int begin_bit, int end_bit,
+                              const unsigned long long* n_dev, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(k_rs_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC_SMEM);
+  if (e != cudaSuccess) return e;
+  MT_COUNT_LAUNCH(1);
+  k_rs_cluster<<<RC_BLOCKS, RC_BS, RC_SMEM, s>>>(keys, vals, n, begin_bit, end_bit, n_dev);
+  return cudaGetLastError();
+}
+
 // one pass: digit [shift, shift + 8) from (k0, v0) to (k1, v1)
 static cudaError_t rs_pass(const uint64_t* k0, const uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n,
                            int shift, void* temp, const unsigned long long* n_dev, bool bal, cudaStream_t s) {
@@ -507,6 +703,7 @@ cudaError_t radix_sort_bits(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, 
                             cudaStream_t s) {
   *in_alt = false;
   if (n <= 1) return cudaSuccess;
+  if (n <= RC_MAX) return rs_cluster(keys, vals, n, begin_bit, end_bit, nullptr, s);
   uint64_t* k0 = keys;
   uint32_t* v0 = vals;
   uint64_t* k1 = keys_alt;
@@ -525,6 +722,7 @@ cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
                              uint32_t* vals_alt, int64_t n, void* temp, cudaStream_t s,
                              const unsigned long long* n_dev) {
   if (n <= 1) return cudaSuccess;
+  if (n <= RC_MAX) return rs_cluster(keys, vals, n, 0, 64, n_dev, s);
   uint64_t* k0 = keys;
   uint32_t* v0 = vals;
   uint64_t* k1 = keys_alt;
