@@ -288,8 +288,10 @@ cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t coun
   // latency; more only lengthen the tail in which a warp waits for its last
   // descents.  Measured: p_20 3 blocks 0.89 ms, 4 0.85, 5 0.84, 6 0.84, 8
   // 0.87; p_24 15.6, 14.4, 13.9, 13.6, 13.4.
-  // q_{l,n} (binary64 pipe, 2 lanes per SM): saturated by 8 warps per SM.
-  if (per_sm > (P.kind == 2 ? 2 : 6)) per_sm = P.kind == 2 ? 2 : 6;
+  // q_{l,n} and the polynomials kept in binary64 (that pipe: 2 lanes per SM)
+  // are saturated by 8 warps per SM (s_{2,16}: 0.72 ms, 1.13 with 24).
+  const int most = P.kind == 2 || !P.fx ? 2 : 6;
+  if (per_sm > most) per_sm = most;
   int64_t grid = (int64_t)device_sm_count() * per_sm;
   const int64_t need = (count + bs - 1) / bs;
   if (grid > need) grid = need;
@@ -313,7 +315,7 @@ cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const u
   const auto kd = P.lcap >= 1 ? &k_descend<true, true> : &k_descend<true, false>;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kd, bs, 0);
   if (e != cudaSuccess) return e;
-  if (per_sm > 6) per_sm = 6;  // as launch_descend
+  if (per_sm > (P.fx ? 6 : 2)) per_sm = P.fx ? 6 : 2;  // as launch_descend
   if (per_sm < 1) per_sm = 1;
   int64_t grid = (int64_t)device_sm_count() * per_sm;
   const int64_t need = (count + bs - 1) / bs;
