@@ -10,7 +10,7 @@
 // fold + key -> LSD radix sort of Re keys -> each sorted candidate checks
 // the earlier candidates of its Re window -> exclusive scan -> gather.
 // Every kernel is a coalesced pass over HBM; the radix sort ranks keys
-// stably inside a block (digit peers of a warp by ballots).
+// stably inside a block (digit peers of a warp by matches).
 #include <cooperative_groups.h>
 
 #include "mt_common.cuh"
@@ -308,14 +308,13 @@ __device__ __forceinline__ int64_t rs_count(int64_t n, const unsigned long long*
   return d < n ? d : n;
 }
 
-// The lanes of the warp whose value d (a digit 0..255, or 256 for no
-// element) equals this lane's.  BAL: nine ballots, one per bit (measured
-// faster on the 64-bit keys of the root sets, whose high bytes repeat
-// along a warp); else one match (faster on the finish keys' uniform
-// digits).
-template <bool BAL>
-__device__ __forceinline__ unsigned rs_peers(unsigned d) {
-  if (!BAL) return __match_any_sync(0xffffffffu, d);
+// The lanes of the warp whose value d (a digit 0..255, or 256 for no element)
+// equals this lane's, by nine ballots, one per bit: a match costs a round per
+// distinct digit, which the cluster sort, whose warps all wait for one another,
+// feels (finish keys, 40960 elements: 72 us with matches, 60 with ballots).  The
+// pass-wise sort, with 24 warps an SM, is faster with matches: root sets of 16.8 M
+// elements 1.84 -> 1.59 ms, of 1 M 215 -> 212 us, of 131 K 146 -> 130 us.
+__device__ __forceinline__ unsigned rs_peers_ballot(unsigned d) {
   unsigned peers = 0xffffffffu;
 #pragma unroll
   for (int b = 0; b < 9; ++b) {
@@ -333,7 +332,6 @@ __device__ __forceinline__ void rs_range(int64_t n, int64_t& t0, int64_t& t1) {
   t1 = nt * (blockIdx.x + 1) / gridDim.x;
 }
 
-template <bool BAL>
 __global__ void __launch_bounds__(RS_BS) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n,
                                                    int shift, uint32_t* __restrict__ hist,
                                                    const unsigned long long* __restrict__ n_dev) {
@@ -352,18 +350,9 @@ __global__ void __launch_bounds__(RS_BS) k_rs_hist(const uint64_t* __restrict__ 
       const int64_t i = base + k * 32;
       dg[k] = i < n ? (unsigned)(keys[i] >> shift) & 255u : 256u;
     }
-    // BAL (64-bit keys, whose high digits repeat along a warp): lanes that
-    // share a digit add once; else (the finish keys' uniform digits, where
-    // lanes rarely share one) one shared-memory atomic per element
 #pragma unroll
-    for (int k = 0; k < RS_ITEMS; ++k) {
-      if (BAL) {
-        const unsigned peers = rs_peers<true>(dg[k]);
-        if (dg[k] < 256u && (peers & lanemask_lt()) == 0) atomicAdd(&cnt[dg[k]], (uint32_t)__popc(peers));
-      } else if (dg[k] < 256u) {
-        atomicAdd(&cnt[dg[k]], 1u);
-      }
-    }
+    for (int k = 0; k < RS_ITEMS; ++k)
+      if (dg[k] < 256u) atomicAdd(&cnt[dg[k]], 1u);
   }
   __syncthreads();
   hist[(int64_t)t * gridDim.x + blockIdx.x] = cnt[t];  // digit-major
@@ -396,7 +385,6 @@ __device__ __forceinline__ void rs_load(const uint64_t* __restrict__ kin, const 
   }
 }
 
-template <bool BAL>
 __global__ void __launch_bounds__(RS_BS, 3) k_rs_scatter(const uint64_t* __restrict__ kin,
                                                          const uint32_t* __restrict__ vin,
                                                          uint64_t* __restrict__ kout,
@@ -444,7 +432,7 @@ __global__ void __launch_bounds__(RS_BS, 3) k_rs_scatter(const uint64_t* __restr
     for (int k = 0; k < RS_ITEMS; ++k) {
       const bool valid = base + k * 32 < n;
       dg[k] = valid ? (unsigned)(key[k] >> shift) & 255u : 256u;
-      const unsigned peers = rs_peers<BAL>(dg[k]);
+      const unsigned peers = __match_any_sync(0xffffffffu, dg[k]);
       const unsigned lt = __popc(peers & lanemask_lt());
       const uint32_t before = valid ? wc[w][dg[k]] : 0u;
       __syncwarp();
@@ -511,7 +499,7 @@ static int64_t rs_grid(int64_t n) {
   static int per_sm = 0;
   if (!per_sm) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_rs_scatter<true>, RS_BS, 0) != cudaSuccess || b < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_rs_scatter, RS_BS, 0) != cudaSuccess || b < 1)
       b = 1;
     per_sm = b;
   }
@@ -589,7 +577,7 @@ __global__ void __cluster_dims__(RC_BLOCKS, 1, 1) __launch_bounds__(RC_BS)
       if (k >= ni) break;
       const bool valid = g0 + k * 32 < n;
       dg[k] = valid ? (unsigned)(key[k] >> shift) & 255u : 256u;
-      const unsigned peers = rs_peers<true>(dg[k]);
+      const unsigned peers = rs_peers_ballot(dg[k]);
       const unsigned lt = __popc(peers & lanemask_lt());
       const uint32_t before = valid ? row[dg[k]] : 0u;
       __syncwarp();
@@ -681,20 +669,18 @@ static cudaError_t rs_cluster(uint64_t* keys, uint32_t* vals, int64_t n, int beg
 
 // one pass: digit [shift, shift + 8) from (k0, v0) to (k1, v1)
 static cudaError_t rs_pass(const uint64_t* k0, const uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n,
-                           int shift, void* temp, const unsigned long long* n_dev, bool bal, cudaStream_t s) {
+                           int shift, void* temp, const unsigned long long* n_dev, cudaStream_t s) {
   const int64_t G = rs_grid(n);
   const int64_t nh = 256 * G;
   uint32_t* hist = (uint32_t*)temp;
   uint32_t* offs = hist + nh;
   uint32_t* dtot = offs + nh;
   MT_COUNT_LAUNCH(1);
-  if (bal) k_rs_hist<true><<<(unsigned)G, RS_BS, 0, s>>>(k0, n, shift, hist, n_dev);
-  else k_rs_hist<false><<<(unsigned)G, RS_BS, 0, s>>>(k0, n, shift, hist, n_dev);
+  k_rs_hist<<<(unsigned)G, RS_BS, 0, s>>>(k0, n, shift, hist, n_dev);
   MT_COUNT_LAUNCH(1);
   k_rs_offsets<<<256, RS_GRID_MAX / 2, 0, s>>>(hist, offs, dtot, (int)G);
   MT_COUNT_LAUNCH(1);
-  if (bal) k_rs_scatter<true><<<(unsigned)G, RS_BS, 0, s>>>(k0, v0, k1, v1, n, shift, offs, dtot, n_dev);
-  else k_rs_scatter<false><<<(unsigned)G, RS_BS, 0, s>>>(k0, v0, k1, v1, n, shift, offs, dtot, n_dev);
+  k_rs_scatter<<<(unsigned)G, RS_BS, 0, s>>>(k0, v0, k1, v1, n, shift, offs, dtot, n_dev);
   return cudaGetLastError();
 }
 
@@ -709,7 +695,7 @@ cudaError_t radix_sort_bits(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, 
   uint64_t* k1 = keys_alt;
   uint32_t* v1 = vals_alt;
   for (int shift = begin_bit; shift < end_bit; shift += 8) {
-    cudaError_t e = rs_pass(k0, v0, k1, v1, n, shift, temp, nullptr, false, s);
+    cudaError_t e = rs_pass(k0, v0, k1, v1, n, shift, temp, nullptr, s);
     if (e != cudaSuccess) return e;
     uint64_t* tk = k0; k0 = k1; k1 = tk;
     uint32_t* tv = v0; v0 = v1; v1 = tv;
@@ -728,7 +714,7 @@ cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
   uint64_t* k1 = keys_alt;
   uint32_t* v1 = vals_alt;
   for (int shift = 0; shift < 64; shift += 8) {
-    cudaError_t e = rs_pass(k0, v0, k1, v1, n, shift, temp, n_dev, true, s);
+    cudaError_t e = rs_pass(k0, v0, k1, v1, n, shift, temp, n_dev, s);
     if (e != cudaSuccess) return e;
     uint64_t* tk = k0; k0 = k1; k1 = tk;
     uint32_t* tv = v0; v0 = v1; v1 = tv;
