@@ -69,10 +69,13 @@ TOL_DD = 1e-20
 
 # ---------------------------------------------------------------------------
 # Algorithmic work per Newton step (flops, FMA = 2), counted from the
-# kernels' arithmetic for an orbit of length m:
+# arithmetic for an orbit of length m:
 #  - binary64 orbit with the scaled derivative: 6 FMA + 1 mul + 1 add per
 #    step, counted 13; the quotient with its range guard, the target or the
-#    update and the stop test 24;
+#    update and the stop test 24.  k_descend, k_walk and k_descend_batch run
+#    this orbit in 64-bit fixed point on the integer pipes: their rate is
+#    given against the binary64 rate that it takes the place of, and may
+#    exceed it;
 #  - binary32 perturbation orbit (mixed tier): 19 flops per step in 12
 #    instructions (two FMA pairs for e, one FMA pair and an FMA/mul for g,
 #    four adds); the binary32 quotient, update and tests 25;
@@ -88,18 +91,37 @@ def newton_flops_fp32(m: int) -> int:
 
 
 def anchor_flops_fp32(m: int) -> int:
-    # the float-float reference orbit the binary32 descent computes per start:
+    # the float-float reference orbit the binary32 descent computes per anchor:
     # per step two TwoProd squares (10 each), a TwoProd product (10), its
     # doubling (2) and three float-float additions (11 each); then P(c0) (two
     # additions) and the jump bound (6)
     return 65 * m + 28
 
 
+# p_n from n = 23 on: one anchor per four starts of the line, and the cubic
+# around it in place of every Newton step's first n - 12 orbit steps
+LONG_MIN, LONG_TAIL, LONG_STARTS = 23, 12, 4
+
+
+def descent_flops_fp32(kind: str, m: int, steps: int, n_starts: int) -> tuple[int, str]:
+    if kind != "hyp" or m < LONG_MIN:
+        a, b = newton_flops_fp32(m), anchor_flops_fp32(m)
+        return steps * a + n_starts * b, "binary32 Newton steps %d x %d flops + float-float anchor orbits %d x %d flops" % (
+            steps, a, n_starts, b)
+    # the cubic and its derivative: d^2 (6), B d and C d^2 (6 each), their sums
+    # (4), the product with d (6), the derivative (10); its coefficients along
+    # the anchor: 13 + 9 + 6 FMA-counted operations a component pair, 44 flops
+    a = 19 * LONG_TAIL + 25 + 38
+    b, na = anchor_flops_fp32(m) + 44 * (m - LONG_TAIL), -(-n_starts // LONG_STARTS)
+    return steps * a + na * b, "binary32 Newton steps %d x %d flops + float-float anchor orbits and series %d x %d flops" % (
+        steps, a, na, b)
+
+
 def finish_flops_fp64(m: int) -> int:
     return 7 * m + 2  # the orbit's value and z - q; the quotient and the tests run in binary32
 
 
-MIX_BATCH = 1 << 23  # starts per launch of the binary32 descent
+MIX_BATCH = 1 << 23  # starts per k_descend_mixed launch the line's per-launch figures refer to
 
 
 def nominal_peak(pipe: str, sm_mhz: float | None) -> float | None:
@@ -126,12 +148,13 @@ def _kernel(name, pipe, flops, ms, launches, peak, peak_nominal, work) -> dict:
 # function of the orbit length m; a bench launch's traffic is this times its
 # own units.  k_descend_mixed reads its start and writes (delta, scale) and
 # the status, its anchor slots staying in L2: 135 + 134 MB per 2^23 starts at
-# p_24, 32.1 B a start.  k_descend (binary64 tier) reads its start (16 B;
+# p_24, 32.1 B a start; with shared anchors (p_n from 23 on) and the far list
+# 548 + 152 MB per 2^24 starts, 41.8 B a start.  k_descend (binary64 tier) reads its start (16 B;
 # 16.8 MB per 2^20 starts).  k_finish_f64: 389 + 141 MB per 4.47 M finishes
 # at p_24, 118.5 B each.  A kernel missing here has changed since its last
 # capture (its traffic is reported as null).
 TRAFFIC = {
-    "k_descend_mixed": (lambda m: 32.1, "start"),
+    "k_descend_mixed": (lambda m: 32.1 if m < LONG_MIN else 41.8, "start"),
     "k_descend": (lambda m: 16, "start"),
     "k_finish_f64": (lambda m: 118.5, "finish"),
 }
@@ -154,22 +177,22 @@ def kernel_rooflines(kind: str, l: int, n: int, stats: list, pk: dict, sm_mhz: f
     if s0.get("ms_k_desc64", 0) > 0 and s0.get("desc_orbit_steps", 0) > 0:  # the batched split
         steps, orb = s0["desc_newton"], s0["desc_orbit_steps"]
         out.append(_kernel("k_descend_batch", "fp64", 13 * orb + 24 * steps, mean("ms_k_desc64"), 1, p64, n64,
-                           "binary64 Newton steps %d: 13 flops x %d orbit steps + 24 x steps" % (steps, orb)))
+                           "Newton steps %d in fixed point (integer pipes, against the binary64 rate): 13 flops x %d orbit steps + 24 x steps" % (steps, orb)))
     elif s0.get("ms_k_desc64", 0) > 0:
         per = 13 * n + 50 * l + 24 if kind == "q" else newton_flops(m)
         # in the mixed tier desc_newton also counts the binary32 steps and the
         # binary64 finish; the binary64 descent kernel ran the tip redo only
         steps = s0["desc_newton"] - s0.get("desc_fp32", 0) - s0.get("finish_newton", 0)
         out.append(_kernel("k_descend_q" if kind == "q" else "k_descend", "fp64", steps * per, mean("ms_k_desc64"),
-                           1, p64, n64, "binary64 Newton steps %d x %d flops" % (steps, per)))
+                           1, p64, n64, "%s Newton steps %d x %d flops" %
+                           ("binary64" if kind == "q" else "fixed-point (integer pipes, against the binary64 rate)", steps, per)))
     if s0.get("ms_k_desc32", 0) > 0:
         steps = s0["desc_fp32"]
         launches = -(-s0["n_starts"] // MIX_BATCH)
-        nst = s0["n_starts"]
-        out.append(_kernel("k_descend_mixed", "fp32", steps * newton_flops_fp32(m) + nst * anchor_flops_fp32(m),
-                           mean("ms_k_desc32"), launches, p32, n32,
-                           "binary32 Newton steps %d x %d flops + float-float anchor orbits %d x %d flops" %
-                           (steps, newton_flops_fp32(m), nst, anchor_flops_fp32(m))))
+        if kind == "hyp" and m >= LONG_MIN:
+            launches = 2  # all starts, then the far list
+        flops, work = descent_flops_fp32(kind, m, steps, s0["n_starts"])
+        out.append(_kernel("k_descend_mixed", "fp32", flops, mean("ms_k_desc32"), launches, p32, n32, work))
     if s0.get("ms_k_finish", 0) > 0:
         steps = s0["finish_newton"]
         out.append(_kernel("k_finish_f64", "fp64", steps * finish_flops_fp64(m), mean("ms_k_finish"), 1, p64, n64,
@@ -177,12 +200,14 @@ def kernel_rooflines(kind: str, l: int, n: int, stats: list, pk: dict, sm_mhz: f
     if s0.get("ms_k_walk", 0) > 0:
         steps = s0["walk_newton"] - s0["seed_newton"]
         if s0["steps_fp32"] > 0:  # binary32 walk sub-steps (the binary64 anchors are not counted)
-            out.append(_kernel("k_walk_mixed", "fp32", steps * newton_flops_fp32(m), mean("ms_k_walk"), 1, p32,
-                               n32, "binary32 walk steps %d x %d flops (anchors not counted)" %
-                               (steps, newton_flops_fp32(m))))
+            long = kind == "hyp" and m >= LONG_MIN  # the series' length varies by turn
+            out.append(_kernel("k_walk_series" if long else "k_walk_mixed", "fp32", steps * newton_flops_fp32(m),
+                               mean("ms_k_walk"), 1, p32, n32, "binary32 walk steps %d x %d flops (anchors not "
+                               "counted%s)" % (steps, newton_flops_fp32(m), "; whole orbits, although a series "
+                                               "takes the place of their first steps" if long else "")))
         else:
             out.append(_kernel("k_walk", "fp64", steps * newton_flops(m), mean("ms_k_walk"), 1, p64, n64,
-                               "binary64 walk steps %d x %d flops" % (steps, newton_flops(m))))
+                               "fixed-point walk steps (integer pipes, against the binary64 rate) %d x %d flops" % (steps, newton_flops(m))))
     mixed = s0.get("desc_fp32", 0) > 0
     for k in out:  # DRAM bytes per launch: measured bytes per unit x this launch's units
         t = TRAFFIC.get(k["kernel"])

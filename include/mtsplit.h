@@ -66,7 +66,7 @@ typedef enum {
 } mt_status;
 
 typedef enum {
-  MT_FP64 = 0,   /* every step in binary64                                      */
+  MT_FP64 = 0,   /* every step in 64 bits: fixed point, binary64 outside its range */
   MT_MIXED = 1,  /* binary32 level-line tracking and early Newton, binary64 finish */
   MT_DD = 2      /* binary64 with double-double for the clustered roots          */
 } mt_precision;

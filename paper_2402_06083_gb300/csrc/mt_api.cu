@@ -247,9 +247,9 @@ bool make_plan(int kind, int l, int n, const mt_options* o, int retry, Plan* pl)
     N0 = std::min<int64_t>(int64_t(1) << 15, Md / 16);
   } else {
     // binary64 in fixed point: the walk is latency-bound with one lane per chunk
-    // until some 2^15 lanes fill the integer pipes, and a seed costs about as
-    // much as 8 sqrt(Md) / 2^8 sub-steps' share of it.  Chunks of 8 sub-steps
-    // up to 2^14 lanes, then as many lanes as sqrt(Md) 2^4 (measured, ms a
+    // until some 2^15 lanes fill the integer pipes, while every lane adds a seed
+    // to lift.  Chunks of 8 sub-steps up to 2^15 of them, then 2^5 sqrt(Md)
+    // chunks, at most 2^18 (half of them run: the upper half; measured, ms a
     // split: p_12 0.455 -> 0.42, p_16 0.62 -> 0.58, p_20 2.37 -> 2.17, p_22 8.1
     // -> 7.0, p_24 32.8 -> 26.2 against 2^14 lanes at most)
     N0 = std::min<int64_t>(int64_t(1) << 15, Md / 8);

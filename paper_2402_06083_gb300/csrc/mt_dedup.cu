@@ -311,7 +311,7 @@ __device__ __forceinline__ int64_t rs_count(int64_t n, const unsigned long long*
 // The lanes of the warp whose value d (a digit 0..255, or 256 for no element)
 // equals this lane's, by nine ballots, one per bit: a match costs a round per
 // distinct digit, which the cluster sort, whose warps all wait for one another,
-// feels (finish keys, 40960 elements: 72 us with matches, 60 with ballots).  The
+// feels (finish keys, 40960 elements: 72 us with matches, 58 with ballots).  The
 // pass-wise sort, with 24 warps an SM, is faster with matches: root sets of 16.8 M
 // elements 1.84 -> 1.59 ms, of 1 M 215 -> 212 us, of 131 K 146 -> 130 us.
 __device__ __forceinline__ unsigned rs_peers_ballot(unsigned d) {
@@ -526,8 +526,8 @@ size_t radix_temp_bytes(int64_t n) {
 //
 // Bound: the two barriers and the chain of a pass (ranks, prefix over the
 // warps, remote counts, digit scan).  Root sets (8 passes): 4097 elements
-// 117 -> 33 us, 16385 141 -> 60, 40960 143 -> 90, where a block's registers and
-// shared memory end; finish keys (5 passes): 4097 83 -> 24, 40960 83 -> 60.
+// 117 -> 33 us, 16385 141 -> 57, 40960 130 -> 86, where a block's registers and
+// shared memory end; finish keys (5 passes): 4097 83 -> 23, 40960 83 -> 58.
 constexpr int RC_BLOCKS = 8;  // the portable cluster size
 constexpr int RC_BS = 1024;
 constexpr int RC_WARPS = RC_BS / 32;
