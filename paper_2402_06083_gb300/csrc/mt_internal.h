@@ -193,9 +193,9 @@ size_t radix_temp_bytes(int64_t n);
 cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt,
                              uint32_t* vals_alt, int64_t n, void* temp, cudaStream_t s,
                              const unsigned long long* n_dev = nullptr);
-// Stable passes on bits [begin_bit, end_bit) only (multiples of 8); the
-// result is in (keys, vals) after an even number of passes, else in the alt
-// buffers (*in_alt = true).
+// Stable passes on bits [begin_bit, end_bit) only (multiples of 8).  *in_alt
+// says where the result is: in the alt buffers after an odd number of passes,
+// else (and for the short lists that one cluster sorts) in (keys, vals).
 cudaError_t radix_sort_bits(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
                             int64_t n, void* temp, int begin_bit, int end_bit, bool* in_alt,
                             cudaStream_t s);
