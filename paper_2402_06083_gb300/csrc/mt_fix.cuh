@@ -16,7 +16,8 @@
 //
 // Numbers.  A coordinate is an integer X of 64 bits, value X 2^-(FB+32), held
 // as two signed limbs h 2^32 + l: FB bits of fraction in the high limb, the
-// components below 2^(30 - FB) (FB = 28: 4, FB = 26: 16).  A product keeps
+// components below 2^(30 - FB) (FB = 28: 4, FB = 26: 16) by one unit of the
+// high limb or more.  A product keeps
 // 2 FB fractional bits: h h exactly plus the cross terms h l + l h, rounded
 // to nearest (the l l term, below a quarter of the last place, is dropped),
 // so a step z^2 + c is off by at most 3/4 2^-2FB in each component: 1.04e-17
@@ -145,15 +146,32 @@ __host__ __device__ __forceinline__ bool fx_below(double x, int E) {
 #endif
   return (unsigned)(hi & 0x7fffffff) < (unsigned)(1023 + E) << 20;
 }
-// every fixed-point operand: |x| < 2^(30 - FB)
+// Every fixed-point operand: |X| < 2^62 - 2^32, so that a limb h, which rounds
+// up, stays below 2^30 and neither 2 h nor a cross term shifted by 31 leaves 32
+// bits.  In value |x| < 2^(30 - FB) less 2^-FB; binary64 points are taken up to
+// 2^(30 - FB) (1 - 2^-21), one unit of their high word below.
 template <int FB>
 __host__ __device__ __forceinline__ bool fx_fits(double x) {
-  return fx_below(x, 30 - FB);
+#ifdef __CUDA_ARCH__
+  const int hi = __double2hiint(x);
+#else
+  long long b;
+  __builtin_memcpy(&b, &x, 8);
+  const int hi = (int)(b >> 32);
+#endif
+  return (unsigned)(hi & 0x7fffffff) < ((unsigned)(1023 + 30 - FB) << 20) - 1u;
 }
 template <int FB>
 __host__ __device__ __forceinline__ bool fx_in(long long X) {
-  const long long L = 1ll << 62;
+  const long long L = (1ll << 62) - (1ll << 32);
   return X > -L && X < L;
+}
+// The same for a product W at 2^-2FB, on its high word (unit 2^(32 - 2FB))
+template <int FB>
+__host__ __device__ __forceinline__ bool fx_out(long long Wr, long long Wi) {
+  constexpr unsigned R = (1u << (FB - 2)) - 1u;
+  const unsigned a = (unsigned)(int)(Wr >> 32) + R, b = (unsigned)(int)(Wi >> 32) + R;
+  return (a > b ? a : b) >= 2u * R;
 }
 
 // w as a float-float, in units of 2^16 (exact to the pair's 48 bits)
@@ -233,7 +251,6 @@ __host__ __device__ __forceinline__ void fx_eval(int m, int lcap, int a8, long l
                                                  const FxTarget& T, FxVal& o) {
   constexpr int S = 32 - FB;   // a product at 2^-2FB to limbs
   constexpr int B = 57;
-  constexpr unsigned R = 1u << (FB - 2);  // the range test on high words: |W| < 2^(30 + FB)
   // c at 2^-2FB and the bits below, which join the cross terms (at 2^-2FB 2^-31)
   const long long CR = (X + (1ll << (S - 1))) >> S, CI = (Y + (1ll << (S - 1))) >> S;
   const long long tr0 = ((X - (CR << S)) << (31 - S)) + (1ll << 30);
@@ -268,7 +285,7 @@ __host__ __device__ __forceinline__ void fx_eval(int m, int lcap, int a8, long l
     Wi = fx_mad(x.h + x.h, y.h, CI) + fx_shr31(ti);
     ++k;
     if (CAP && k == lcap) { cwr = Wr; cwi = Wi; cdu = Du; cdv = Dv; cex = Ex; }
-    return k >= m || (((unsigned)fx_hi(Wr) + R) | ((unsigned)fx_hi(Wi) + R)) >= 2u * R;
+    return k >= m || fx_out<FB>(Wr, Wi);
   };
   if (m > 1) {
     for (;;) {
@@ -395,10 +412,9 @@ __host__ __device__ __forceinline__ void fx_eval(int m, int lcap, int a8, long l
   o.ii = ff_neg(ff_mul(di, r));
 }
 
-#ifdef __CUDACC__
 // w 2^-2FB in binary32, to its full relative precision (two exact halves)
 template <int FB>
-__device__ __forceinline__ float fx_to_f32(long long w) {
+__host__ __device__ __forceinline__ float fx_to_f32(long long w) {
   return fmaf((float)fx_hi(w), fx_pow2f(32 - 2 * FB), (float)(unsigned)w * fx_pow2f(-2 * FB));
 }
 
@@ -407,10 +423,9 @@ __device__ __forceinline__ float fx_to_f32(long long w) {
 // orbit leaves the fixed range before its last step.  The value alone is a
 // third of fx_eval's step; its binary32 companions run beside it.
 template <int FB>
-__device__ __forceinline__ bool fx_value_d32_k(int m, long long X, long long Y, long long& Wr, long long& Wi,
+__host__ __device__ __forceinline__ bool fx_value_d32_k(int m, long long X, long long Y, long long& Wr, long long& Wi,
                                                float& dr, float& di, float& kr, float& ki) {
   constexpr int S = 32 - FB;
-  constexpr unsigned R = 1u << (FB - 2);
   const long long CR = (X + (1ll << (S - 1))) >> S, CI = (Y + (1ll << (S - 1))) >> S;
   const long long tr0 = ((X - (CR << S)) << (31 - S)) + (1ll << 30);
   const long long ti0 = ((Y - (CI << S)) << (31 - S)) + (1ll << 30);
@@ -431,7 +446,7 @@ __device__ __forceinline__ bool fx_value_d32_k(int m, long long X, long long Y, 
     const float ndr = fmaf(tfr, dzr, fmaf(-tfi, dzi, 1.f));
     const float ndi = fmaf(tfr, dzi, tfi * dzr);
     dzr = ndr; dzi = ndi; ur = nur; ui = nui;
-    in = in && (((unsigned)fx_hi(wr) + R) | ((unsigned)fx_hi(wi) + R)) < 2u * R;
+    in = in && !fx_out<FB>(wr, wi);
     const int nyh = -y.h;
     const long long tr = fx_mad(nyh, y.l, fx_mad(x.h, x.l, tr0));
     const long long ti = fx_mad(x.l, y.h, fx_mad(x.h, y.l, ti0));
@@ -452,7 +467,6 @@ __device__ __forceinline__ bool fx_value_d32_k(int m, long long X, long long Y, 
   ki = fmaf(ai, cr2, -ar * ci2) * inv;
   return in;
 }
-#endif
 
 // (a + ib) (c + id) 2^sc
 __host__ __device__ __forceinline__ void fx_cmul(ff a, ff b, ff c, ff d, int sc, ff& qr, ff& qi) {
