@@ -82,20 +82,36 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
   int m = 1, lcap = -1, cap = 20, outcome = -1;
   unsigned long long steps = 0, orbit = 0, nconv = 0, ndiv = 0, nto = 0;
   bool drained = false;
+  __shared__ int64_t axis_buf[4][64];
+  int64_t* abuf = axis_buf[threadIdx.x >> 5];
+  unsigned na = 0;
+  auto axis = [&]() {
+    int64_t i;
+    if (axis_pop(abuf, na, i)) {
+      const PolyDev& P = E[seg[i]].P;
+      cand[i] = axis_step(P.m, P.lcap, cand[i]);
+    }
+  };
   for (;;) {
     // as k_descend: written and refilled together once DESC_REFILL lanes wait
     const unsigned running = __ballot_sync(0xffffffffu, idx >= 0 && idx < count && outcome < 0);
     const unsigned wait = __popc(__ballot_sync(0xffffffffu, idx < 0 || outcome >= 0));
     if (wait >= DESC_REFILL || running == 0u) {
+      bool near = false;
+      const int64_t at = idx;
       if (outcome >= 0) {
-        cand[idx] = descent_point(d);
-        status[idx] = (uint8_t)outcome;
+        const double2 z = descent_point(d);
+        cand[at] = z;
+        near = outcome == 0 && d.fx && fx_below(z.y, AXIS_EXP);
+        status[at] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
         nto += outcome == 2;
         outcome = -1;
         idx = -1;
       }
+      axis_push(abuf, na, near, at);
+      if (na >= 32u) axis();
       const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
       if (need) {
         unsigned long long base = 0;
@@ -129,6 +145,7 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
       orbit += (unsigned)m;
     }
   }
+  if (na) axis();
   warp_add_u64(&ctr->desc_newton, steps);
   warp_add_u64(&ctr->desc_orbit, orbit);
   warp_add_u64(&ctr->n_conv, nconv);

@@ -54,6 +54,45 @@ static __device__ __noinline__ double2 newton_step_f64(int m, int lcap, double2 
   return make_double2(z.x - qr, z.y - qi);
 }
 
+// Roots next to the real axis.  A fixed-point coordinate is off by some 2e-18
+// however small it is; in binary64 the error of a small Im shrinks with it (and
+// at the root 0 that of Re as well).  rms of Im over the roots of p_20 with |Im|
+// below 1e-6: 1.4e-18 fixed, 1.8e-19 binary64; in [1e-6, 1e-4) 2.2e-18 and
+// 4.7e-19; from 1e-4 on the fixed point is the closer (2.3e-18 and 7.3e-18).
+// So the components below 2^-13 of a converged point are taken from one more
+// step with the value in binary64 (P' in binary32: the step is ~1e-16, its
+// relative error of 1e-6 is nothing); the others keep the fixed point's digits.
+constexpr int AXIS_EXP = -13;
+static __device__ __noinline__ double2 axis_step(int m, int lcap, double2 z) {
+  double vr, vi;
+  float dr, di, qr, qi;
+  orbit_f64_d32(m, lcap, z.x, z.y, vr, vi, dr, di);
+  if (!cdiv_f32s(f32_trunc(vr), f32_trunc(vi), dr, di, qr, qi)) return z;
+  if (fx_below(z.x, AXIS_EXP)) z.x -= f64_of_f32(qr);
+  if (fx_below(z.y, AXIS_EXP)) z.y -= f64_of_f32(qi);
+  return z;
+}
+// A warp gathers such points (their indices in cand) and steps 32 of them
+// together, since a binary64 step costs it the same for one.  buf: its 64
+// entries of shared memory; n: entries waiting (warp-uniform).
+template <class T>
+__device__ __forceinline__ void axis_push(T* buf, unsigned& n, bool mine, T at) {
+  const unsigned b = __ballot_sync(0xffffffffu, mine);
+  if (mine) buf[n + __popc(b & lanemask_lt())] = at;
+  n += __popc(b);
+}
+// the last (up to 32) entries: true for the lanes that received one (*at)
+template <class T>
+__device__ __forceinline__ bool axis_pop(const T* buf, unsigned& n, T& at) {
+  __syncwarp();  // the entries, and the candidates they name, are written
+  const unsigned c = n < 32u ? n : 32u;
+  n -= c;
+  const bool mine = (threadIdx.x & 31) < c;
+  if (mine) at = buf[n + (threadIdx.x & 31)];
+  __syncwarp();  // read before the next push
+  return mine;
+}
+
 // One Newton step and its outcome: -1 go on, 0 converged, 1 divergent, 2 cap.
 template <bool CAP>
 __device__ __forceinline__ int descent_step(int m, int lcap, Descent& d, float tol2, int cap) {

@@ -29,6 +29,7 @@
 // its binary64 finishing steps.  The chunk-end check of the walk and the
 // count check catch any tracking failure, and the host then repeats the
 // split in plain binary64.
+#include "mt_descent.cuh"
 #include "mt_fix.cuh"
 #include "mt_levelline.cuh"
 #include "mt_pert.cuh"
@@ -1106,7 +1107,8 @@ __global__ void k_finish_list(int64_t count, const uint32_t* __restrict__ head, 
 // binary64 (the polynomials kept there).  Bound: the integer multiply-add
 // pipe (56 %) and issue (70 %); in binary64 that pipe's 3 FMA a step, 16 clocks
 // a warp each, with the heads outside the line repeating six steps.  p_24, 4.5 M
-// heads: 0.865 -> 0.273 ms (p_28 15.1 -> 4.65; not taken there, FIN_FX_MAXM).
+// heads: 0.865 -> 0.305 ms, 0.03 of it the binary64 step of the small imaginary
+// parts (axis_step) (p_28 15.1 -> 4.65 without it; not taken there, FIN_FX_MAXM).
 constexpr int FIN_FB = 28;
 constexpr unsigned FIN_REFILL = 6;
 template <bool FX>
@@ -1128,17 +1130,30 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
   bool have = false;
   bool drained = false;  // warp-uniform: the list is handed out
   unsigned s64 = 0;
+  __shared__ uint32_t axis_buf[FX ? 4 : 1][64];
+  uint32_t* abuf = axis_buf[FX ? threadIdx.x >> 5 : 0];
+  unsigned na = 0;
+  auto axis = [&]() {
+    uint32_t i;
+    if (axis_pop(abuf, na, i)) cand[i] = axis_step(P.m, P.lcap, cand[i]);
+  };
   for (;;) {
     const unsigned wait = __ballot_sync(0xffffffffu, outcome >= 0);
     if (__popc(wait) >= (drained ? 32u : FX ? FIN_REFILL : 1u)) {
+      bool near = false;
       if (have && outcome >= 0) {
         if (FX) {
           zx = fx_to_f64<FIN_FB>(X);
           zy = fx_to_f64<FIN_FB>(Y);
+          near = outcome == 0 && fx_below(zy, AXIS_EXP);
         }
         cand[at] = make_double2(zx, zy);
         status[at] = (uint8_t)outcome;
         have = false;
+      }
+      if (FX) {
+        axis_push(abuf, na, near, at);
+        if (na >= 32u) axis();
       }
       if (drained) break;
       unsigned long long b0 = 0;
@@ -1230,6 +1245,7 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
       prev2 = s2;
     }
   }
+  if (FX && na) axis();
   warp_add_u64(&ctr->desc_newton, s64);
   warp_add_u64(&ctr->finish_newton, s64);
 }

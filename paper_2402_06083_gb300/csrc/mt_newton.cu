@@ -39,6 +39,13 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
   Descent d{0, 0, 16.f, 3.0e38f, 0, false, true};
   unsigned steps = 0, nconv = 0, ndiv = 0, nto = 0;
   bool drained = false;  // warp-uniform
+  __shared__ int64_t axis_buf[4][64];
+  int64_t* abuf = axis_buf[threadIdx.x >> 5];
+  unsigned na = 0;
+  auto axis = [&]() {
+    int64_t i;
+    if (axis_pop(abuf, na, i)) cand[i] = axis_step(P.m, P.lcap, cand[i]);
+  };
   for (;;) {
     // Lanes that finished are written and refilled together, once DESC_REFILL
     // of them wait or none is running: both cost a pass of the warp however
@@ -47,8 +54,11 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
     const unsigned running = __ballot_sync(0xffffffffu, active0);
     const unsigned wait = __popc(__ballot_sync(0xffffffffu, idx < 0 || outcome >= 0));
     if (wait >= DESC_REFILL || running == 0u) {
+      bool near = false;
       if (outcome >= 0) {
-        cand[at] = descent_point(d);
+        const double2 z = descent_point(d);
+        cand[at] = z;
+        near = outcome == 0 && d.fx && fx_below(z.y, AXIS_EXP);
         status[at] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
@@ -56,6 +66,8 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
         outcome = -1;
         idx = -1;
       }
+      axis_push(abuf, na, near, at);
+      if (na >= 32u) axis();
       const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
       if (need) {
         unsigned long long base = 0;
@@ -82,6 +94,7 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
       ++steps;
     }
   }
+  if (na) axis();
   warp_add_u64(&ctr->desc_newton, steps);
   if (!LIST) {  // a list's outcomes are counted where it joins the others
     warp_add_u64(&ctr->n_conv, nconv);
