@@ -125,9 +125,12 @@ __device__ __forceinline__ int descent_step(int m, int lcap, Descent& d, float t
     descent_set(d, z.x, z.y);
   }
   float ax, ay;
-  if (d.wide) {  // inf or NaN stays so
-    ax = f32_trunc(__longlong_as_double(d.X));
-    ay = f32_trunc(__longlong_as_double(d.Y));
+  bool lost = false;
+  if (d.wide) {  // beyond binary32 (2^64 for |z|^2) inf, as the radius of such a start
+    const double2 z = descent_point(d);
+    lost = !finite2(z.x, z.y);
+    ax = f32_trunc(z.x);
+    ay = f32_trunc(z.y);
   } else {
     ax = (float)fx_hi(d.X) * (1.f / (1 << FXB));
     ay = (float)fx_hi(d.Y) * (1.f / (1 << FXB));
@@ -136,7 +139,7 @@ __device__ __forceinline__ int descent_step(int m, int lcap, Descent& d, float t
   int outcome = -1;
   const float fl = (1.f + fabsf(ax) + fabsf(ay)) * 3.552713678800501e-15f;  // 16 ulp of binary64
   const float z2 = fmaf(ax, ax, ay * ay);
-  if (!(z2 <= d.rdiv2) || z2 > 3.0e38f) outcome = 1;
+  if (lost || !(z2 <= d.rdiv2)) outcome = 1;
   else if (s2 < tol2) outcome = 0;  // the step that met tol also squared the error
   // binary64 rounding floor: steps stopped shrinking within a few ulp of z
   // (between two close roots Newton also stalls, at |step| ~ their

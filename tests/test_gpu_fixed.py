@@ -61,3 +61,23 @@ def test_descents_from_inside_and_outside_the_range(mt, kind, n, l):
     for c in conv[:: max(1, conv.size // 200)]:
         _, disp = oracle.polish(kind, n, c, steps=3, l=l)
         assert disp <= 4e-16 * abs(c) + 4e-16, (c, disp)
+
+
+@pytest.mark.parametrize("kind,n,l,exps", [("hyp", 1, 0, (18, 19, 20, 38, 100, 150, 300)), ("hyp", 2, 0, (18, 20, 39, 100)),
+                                           ("hyp", 3, 0, (18, 20, 39, 60)), ("hyp", 4, 0, (18, 20, 30)),
+                                           ("mis", 1, 2, (18, 20, 39, 100)), ("mis", 2, 2, (18, 20, 39, 60))])
+def test_descents_from_far_away(mt, kind, n, l, exps):
+    """From |z0| so large that z0 alone decides (P ~ z^d), a Newton step is
+    (1 - 1/d) z: 20 of them (the cap), no long jump; p_1 = z is at its root
+    after one.  Relative error 20 binary64 steps of a few roundings each, and the
+    next term of P, at most 2 / |z| a step and so 4 d over the last point."""
+    z = np.array([s * 10.0 ** e for e in exps for s in (1, -1, 1j, 0.6 - 0.8j)])
+    out, status, _ = mt.descend(kind, n, _t(z), l=l)
+    out, status = out.cpu().numpy(), status.cpu().numpy()
+    d = 2 ** (n - 1) if kind == "hyp" else 2 ** (l + n - 2)
+    if d == 1:
+        assert np.all(status == 0) and np.all(out == 0)
+    else:
+        assert np.all(status == 2)
+        err = np.abs(out / (z * (1 - 1 / d) ** 20) - 1)
+        assert np.all(err < 20 * 32 * 2.0 ** -53 + 4 * d / np.abs(out))
