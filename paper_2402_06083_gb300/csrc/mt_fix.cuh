@@ -374,9 +374,11 @@ __host__ __device__ __forceinline__ void fx_eval(int m, int lcap, int a8, long l
     float IUs = IU;
     if (k < m) {
       const int r = m - k;
-      // |P| ~ |p_k|^(2^r): past binary64's range from 2^1024 on
-      const float lz = log2f(fmaxf(fabsf(zr.hi), fabsf(zi.hi)));
-      o.over = r > 6 || lz * (float)(1 << r) >= 1024.f;
+      // |P| ~ |p_k|^(2^r) and |P'| ~ |p'_k| 2^r |p_k|^(2^r - 1): past binary64's
+      // range from 2^1024 on
+      const float lz = 0.5f * log2f(fmaf(zr.hi, zr.hi, zi.hi * zi.hi));
+      const float ld = log2f(fmaxf(fabsf(dr.hi), fabsf(di.hi))) + (float)(ed + r);
+      o.over = r > 6 || lz * (float)(1 << r) >= 1024.f || ld + lz * (float)((1 << r) - 1) >= 1024.f;
       IUs = 5.421010862427522e-20f;  // n = p_k 2^-64; the target and p_lcap no longer count
       o.sc += 64 - 16 + 2 * FB - r;
     } else if (CAP && lcap >= 1) {

@@ -7,6 +7,7 @@ import ctypes
 import os
 import shutil
 import subprocess
+from decimal import Context, Decimal
 from fractions import Fraction
 
 import numpy as np
@@ -144,3 +145,39 @@ def test_value_next_to_the_end_of_the_range(fx, m):
         seen += 1
         assert abs(v[0] - float(z[0])) + abs(v[1] - float(z[1])) <= 2 * tol, (x, y)
     assert seen > 20
+
+
+def _log2_exact(m, x, y):
+    """log2 of the larger component of P and of P' of p_m, past any range."""
+    C = Context(prec=40, Emax=10 ** 9, Emin=-10 ** 9)
+    add, sub, mul = C.add, C.subtract, C.multiply
+    x, y, zero = Decimal(x), Decimal(y), Decimal(0)
+    zr, zi, dr, di = x, y, Decimal(1), zero
+    for _ in range(2, m + 1):
+        tr, ti = sub(mul(zr, dr), mul(zi, di)), add(mul(zr, di), mul(zi, dr))
+        dr, di = add(add(tr, tr), 1), add(ti, ti)
+        zr, zi = add(sub(mul(zr, zr), mul(zi, zi)), x), add(mul(2, mul(zr, zi)), y)
+    big = lambda a, b: float(C.ln(max(abs(a), abs(b)))) / np.log(2.0)
+    return big(zr, zi), big(dr, di)
+
+
+@pytest.mark.parametrize("m", [10, 11])
+def test_orbits_past_the_range_of_binary64(fx, m):
+    """Reported where P or P' reaches 2^1024, whichever comes first (a component
+    of a value of that size may be half a bit smaller: a band of one bit at
+    either side is left out)."""
+    rng = np.random.default_rng(m)
+    q = (ctypes.c_double * 2)()
+    seen = [0, 0, 0]
+    for _ in range(6000):
+        r, a = rng.uniform(2.0, 5.6), rng.uniform(0, 2 * np.pi)
+        x, y = float(r * np.cos(a)), float(r * np.sin(a))
+        got = fx.fx_newton(28, m, 0, x, y, q)
+        if got < 0:
+            continue
+        lp, ld = _log2_exact(m, x, y)
+        if abs(max(lp, ld) - 1024) < 1:
+            continue
+        assert got == (1 if max(lp, ld) > 1024 else 0), (x, y, lp, ld)
+        seen[0 if max(lp, ld) < 1024 else 1 if lp > 1024 else 2] += 1
+    assert min(seen) >= 5, seen
