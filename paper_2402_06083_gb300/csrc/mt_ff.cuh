@@ -51,4 +51,18 @@ __host__ __device__ __forceinline__ ff ff_rcp(ff a) {
   return ff_norm(r, r * e);
 }
 
+// The square of the radius within which A d + B d^2 + C d^3 stands for p_K
+// around an anchor: |C| rho^2 = 1e-4 |A| and |B| rho = 1e-2 |A| (in the
+// maximum norm: C ~ A^3 passes 2^64, its square binary32's range).  Negative,
+// so that not even the anchor itself is within it, where a coefficient leaves
+// binary32's range.
+__host__ __device__ __forceinline__ float series_rho2(float Ax, float Ay, float Bx, float By, float Cx, float Cy) {
+  const float a = fmaxf(fabsf(Ax), fabsf(Ay)), b = fmaxf(fabsf(Bx), fabsf(By)), c = fmaxf(fabsf(Cx), fabsf(Cy)),
+              ab = a / b;
+  const float r = fminf(1e-4f * a / c, 1e-4f * ab * ab);
+  // 0 only where all six are finite (fmaxf passes over a NaN)
+  const float f = 0.f * (((Ax + Ay) + (Bx + By)) + (Cx + Cy));
+  return f == 0.f && c < 1e37f && r > 0.f ? r : -1.f;
+}
+
 }  // namespace mt

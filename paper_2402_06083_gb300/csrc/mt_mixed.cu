@@ -609,15 +609,8 @@ __device__ __forceinline__ void anchor_orbit(const PolyDev& P, int K, double2 c0
   }
   const ff vx = ff_add(zx, capx), vy = ff_add(zy, capy);
   w.zv[j] = make_float4(vx.hi, vy.hi, vx.lo, vy.lo);
-  // rho^2; no bound where nothing is skipped, 0 (never valid) out of binary32's range
-  float rho2 = 3.0e38f;
-  if (K > 1) {
-    // (in the maximum norm: C ~ A^3 passes 2^64, its square binary32's range)
-    const float a = fmaxf(fabsf(Ax), fabsf(Ay)), b = fmaxf(fabsf(Bx), fabsf(By)), c = fmaxf(fabsf(Cx), fabsf(Cy)),
-                ab = a / b;
-    rho2 = fminf(1e-4f * a / c, 1e-4f * ab * ab);
-    if (!(c < 1e37f && rho2 > 0.f)) rho2 = 0.f;
-  }
+  // rho^2; no bound where nothing is skipped
+  const float rho2 = K > 1 ? series_rho2(Ax, Ay, Bx, By, Cx, Cy) : 3.0e38f;
   // long jump (as in k_descend: |c| > max(4, 2|c0|)); |delta| beyond rdel implies it
   const float r0 = sqrtf(fmaf(cx.hi, cx.hi, cy.hi * cy.hi)) * 1.0001f;
   w.zab[j] = make_float4(Ax, Ay, Bx, By);

@@ -37,6 +37,7 @@ extern "C" int fx_newton(int fb, int m, int lcap, double x, double y, double* q)
   if (fb == 27) return lcap < 1 ? newton<27, false>(m, lcap, x, y, q) : newton<27, true>(m, lcap, x, y, q);
   return lcap < 1 ? newton<26, false>(m, lcap, x, y, q) : newton<26, true>(m, lcap, x, y, q);
 }
+extern "C" float rho2(const float* k) { return series_rho2(k[0], k[1], k[2], k[3], k[4], k[5]); }
 extern "C" int fx_value(int m, double x, double y, double* v) {  // FB = 28
   if (!(fx_fits<28>(x) && fx_fits<28>(y))) return -1;
   long long wr, wi;
@@ -63,6 +64,8 @@ def fx(tmp_path_factory):
     L = ctypes.CDLL(lib)
     L.fx_newton.argtypes = [ctypes.c_int] * 3 + [ctypes.c_double] * 2 + [ctypes.c_void_p]
     L.fx_value.argtypes = [ctypes.c_int] + [ctypes.c_double] * 2 + [ctypes.c_void_p]
+    L.rho2.argtypes = [ctypes.c_void_p]
+    L.rho2.restype = ctypes.c_float
     return L
 
 
@@ -181,3 +184,17 @@ def test_orbits_past_the_range_of_binary64(fx, m):
         assert got == (1 if max(lp, ld) > 1024 else 0), (x, y, lp, ld)
         seen[0 if max(lp, ld) < 1024 else 1 if lp > 1024 else 2] += 1
     assert min(seen) >= 5, seen
+
+
+def test_series_out_of_range_holds_nowhere(fx):
+    """The radius of the mixed descents' series: that of its definition, and
+    none at all (the anchor's own d = 0 lies outside) for coefficients that
+    binary32 cannot hold."""
+    inf, nan = float("inf"), float("nan")
+    f = lambda *k: fx.rho2((ctypes.c_float * 6)(*k))
+    assert abs(f(2.0 ** 30, 0, 2.0 ** 50, 0, 2.0 ** 80, 0) / (1e-4 * 2.0 ** -50) - 1) < 1e-6
+    assert abs(f(0, -2.0 ** 30, 0, 2.0 ** 60, 1.0, 0) / (1e-4 * 2.0 ** -60) - 1) < 1e-6
+    for C in ((1e37, 0), (0, -2e37), (inf, 0), (nan, 0), (0, nan), (nan, nan), (-inf, nan)):
+        assert not 0.0 <= f(2.0 ** 41, 0, 2.0 ** 80, 0, *C), C
+    for AB in ((inf, 0, 1, 0), (nan, nan, 1, 0), (1, 0, inf, 0), (1, 0, nan, nan), (2.0 ** 41, 0, 3e38, 3e38)):
+        assert not 0.0 <= f(*AB, 1.0, 0.0), AB
