@@ -710,6 +710,13 @@ constexpr int DM_BS = 128;     // threads per block of the binary32 descent
 constexpr int DM_REFILL = 11;
 constexpr int DM_MAX_WARPS = 16384;  // warp slots of the anchor buffer (grids are capped to fit)
 constexpr int DM_TAIL = 12;
+constexpr int DM_GSH = 2;  // log2 of the starts that share an anchor
+// The work queue and the start indices are 32-bit.  A warp takes ranges of up to
+// 32 << DM_GSH starts until one begins past the last start, so the queue ends
+// below count + (warps + 1) ranges, which must not wrap: a wrapped queue would
+// hand out its starts again, without an end.
+constexpr int64_t DM_MAX_COUNT = 0xffd00000ll;
+static_assert(DM_MAX_COUNT + (DM_MAX_WARPS + 1ll) * (32ll << DM_GSH) <= (1ll << 32), "the queue wraps");
 template <bool CAP, int MC, bool LIST>
 __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, int Kr, int gsh,
                                                          const double2* __restrict__ starts, int64_t cnt,
@@ -1347,7 +1354,7 @@ static cudaError_t launch_dm(DescMixedFn kern, const PolyDev& P, int K, int gsh,
   const int64_t need = (count + bs - 1) / bs;
   if (grid > need) grid = need;
   if (grid > DM_MAX_WARPS / (bs / 32)) grid = DM_MAX_WARPS / (bs / 32);
-  unsigned* q = (unsigned*)&ctr->queue_head;  // 32 bits: the last ranges end below 2^32
+  unsigned* q = (unsigned*)&ctr->queue_head;
   if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess) return e;
   MT_COUNT_LAUNCH(1);
   if ((e = ktimer_begin(KS_DESC32, s)) != cudaSuccess) return e;
@@ -1360,7 +1367,7 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
                                  double2* cand, uint8_t* status, void* anchors, const FinishScratch& fin,
                                  DevCounters* ctr, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
-  if (P.m > MIX_MAXM || count > 0xfff00000ll) return cudaErrorInvalidValue;  // 32-bit queue and list
+  if (P.m > MIX_MAXM || count > DM_MAX_COUNT) return cudaErrorInvalidValue;
   const int bs = DM_BS;
   cudaError_t e = cudaSuccess;
   float2* wbuf = (float2*)anchors;
@@ -1371,7 +1378,7 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
     // (s_{6,12}: none of 7 levels without, 3 with).
     const bool shared = P.kind == 0 && P.m >= MIX_LONG;
     const int K = shared ? P.m - DM_TAIL : 1;
-    const int gsh = shared ? 2 : 0;
+    const int gsh = shared ? DM_GSH : 0;
     uint32_t* far = fin.pos;  // free until the finish's scan
     unsigned long long* nfar = fin.nheads;
     if ((e = cudaMemsetAsync(nfar, 0, sizeof(*nfar), s)) != cudaSuccess) return e;
