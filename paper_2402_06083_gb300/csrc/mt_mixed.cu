@@ -576,6 +576,12 @@ __device__ __forceinline__ WarpSlot warp_slot(float2* wbuf, int rows, unsigned w
   w.za = b + SLOT_EXTRA;
   return w;
 }
+// Starts left of this go on the far list at once, and so get an anchor each.  By
+// the left tip single pairs of real roots lie 5e-4 of the starts' spacing apart
+// (p_24: 2.1e-13 at -2 + 8.8e-7), where binary32 around a start's own orbit just
+// tells them apart and around a neighbour's does not: of 5000 levels of p_24, 276
+// missed a root and had the split repeated in binary64, 144 with an anchor a start.
+constexpr float DM_TIP = -1.999f;
 template <bool CAP, int MC>
 __device__ __forceinline__ void anchor_orbit(const PolyDev& P, int K, double2 c0, const WarpSlot& w, unsigned j) {
   const int m = MC > 0 ? MC : P.m;
@@ -609,8 +615,8 @@ __device__ __forceinline__ void anchor_orbit(const PolyDev& P, int K, double2 c0
   }
   const ff vx = ff_add(zx, capx), vy = ff_add(zy, capy);
   w.zv[j] = make_float4(vx.hi, vy.hi, vx.lo, vy.lo);
-  // rho^2; no bound where nothing is skipped
-  const float rho2 = K > 1 ? series_rho2(Ax, Ay, Bx, By, Cx, Cy) : 3.0e38f;
+  // rho^2; no bound where nothing is skipped, none for the starts at the tip
+  const float rho2 = K <= 1 ? 3.0e38f : cx.hi < DM_TIP ? -1.f : series_rho2(Ax, Ay, Bx, By, Cx, Cy);
   // long jump (as in k_descend: |c| > max(4, 2|c0|)); |delta| beyond rdel implies it
   const float r0 = sqrtf(fmaf(cx.hi, cx.hi, cy.hi * cy.hi)) * 1.0001f;
   w.zab[j] = make_float4(Ax, Ay, Bx, By);
@@ -701,7 +707,8 @@ __device__ __forceinline__ void pert_eval_series(const PolyDev& P, int Kr, const
 // at compile time (p_n), else 0.
 //
 // Bound by issue (80 %) and the binary32 pipe (50 %).  p_28, 268 M starts: 53.4
-// ms with an anchor a start and every orbit step, 29.1 now; p_24 2.93 -> 1.84.
+// ms with an anchor a start and every orbit step, 29.6 now (29.0 if the starts
+// left of DM_TIP shared too); p_24 2.93 -> 1.86.
 constexpr int DM_BS = 128;     // threads per block of the binary32 descent
 // Idle lanes that trigger a refill, and orbit steps after the series: the
 // refill's pass (the end's record, the next orbit's copy) costs about a third of a

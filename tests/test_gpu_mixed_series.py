@@ -36,3 +36,14 @@ def test_first_attempt_finds_every_root(mt, n, kw):
     assert st["prec_used"] == 1 and st["n_roots"] == 2 ** (n - 1)
     a, b = r.roots.cpu().numpy(), mt.split_hyperbolic(n).roots.cpu().numpy()
     assert np.max(np.abs(a - b)) < 1e-13
+
+
+@pytest.mark.parametrize("level", [5.935373876248844, 5.287923032490966, 5.828942694987802, 5.27979241373518,
+                                   5.224064323734339, 5.820812076232031, 5.942318253715001, 5.212828084963434])
+def test_close_pairs_at_the_tip_are_told_apart(mt, level):
+    """Levels of p_24 whose line sends two or three starts to one root of a real
+    pair at the left tip, 2e-13 to 5e-12 apart where starts lie 4e-10 to 3e-9
+    apart: around an anchor of its own each start reaches its root, around a
+    neighbour's one of the pair was missed."""
+    st = mt.split_hyperbolic(24, "mixed", max_retries=-1, check_status=False, lambda0=level).stats
+    assert st["n_roots"] == st["n_cert_pass"] == 2 ** 23
