@@ -769,10 +769,9 @@ def measure(b: Bench, name: str, steps: int, warmup: int, pk: dict, peak_source:
                 "ms_per_step": e2e_s * 1e3,
                 "call_ms": [round(x, 1) for x in getattr(b, "e2e_step_ms", [])],
                 "copy_ms": [round(x, 1) for x in getattr(b, "e2e_copy_ms", [])],
-                "note": "the input is the integer n (no device input); each step's sorted roots (and low parts) "
-                        "are copied to pinned host memory inside the timed loop, on a second stream while the "
-                        "next step splits into the other of two output buffers; the time ends when the last "
-                        "copy has landed"},
+                "note": "the input is the integer n (no device input); each step's roots (and low parts) are copied to "
+                        "pinned host memory in the timed loop, on a second stream while the next step splits into "
+                        "the other of two buffers; the time ends when the last copy has landed"},
         "roofline": roofline_of(kern, peak_source), "kernels": kern,
         "gpu_launches": int(sum(s["n_launches"] for s in stats)), "clocks": clocks,
         "detail": {k: s0.get(k) for k in (
@@ -807,6 +806,66 @@ def measure(b: Bench, name: str, steps: int, warmup: int, pk: dict, peak_source:
     return rec
 
 
+def sig(x, digits: int = 6):
+    """Every number of a record to 'digits' significant digits."""
+    if isinstance(x, dict):
+        return {k: sig(v, digits) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [sig(v, digits) for v in x]
+    return float("%.*g" % (digits, x)) if isinstance(x, float) else x
+
+
+def kernel_summary(kernels: list) -> list:
+    return [{k: x[k] for k in ("kernel", "pipe", "frac", "ms_per_launch", "launches")} for x in kernels]
+
+
+def error_summary(e: dict) -> dict:
+    return {k: e[k] for k in ("max_abs", "max_abs_fp64_roots", "max_abs_dd_roots", "tol_fp64", "tol_dd", "checked_fp64",
+                              "checked_dd", "roots", "within_tol") if k in e}
+
+
+def line_of(rec: dict, subs: dict, steps: int, warmup: int, world: int, pk: dict) -> dict:
+    """The printed line: the main record with its headline roofline, and a
+    summary of each other workload.  Kept to a few thousand characters, so that
+    whatever reads the last lines of a run's output gets it whole; --record has
+    the rest."""
+    keep = ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step", "note")
+    line = {
+        "metric": METRIC, "value": rec["value"], "unit": "roots/s", "n_gpus": world, "steps": steps,
+        "warmup": warmup, "ms_per_step": rec["ms_per_step"], "higher_is_better": True,
+        "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic (inputs fixed by n)",
+        "config": {"workload": rec["workload"], "precision": rec["precision"],
+                   "l2": "flushed between timed steps (256 MB write)",
+                   "parallelism": "replicas" if world > 1 else "single GPU"},
+        "e2e": {k: rec["e2e"][k] for k in keep}, "gpu_launches": rec["gpu_launches"], "clocks": rec["clocks"],
+        "roofline": rec["roofline"], "kernels": kernel_summary(rec["kernels"]),
+        "peaks": {"fp64_tflops": pk["fp64"], "fp32_tflops": pk["fp32"]},
+        "detail": {k: v for k, v in rec["detail"].items() if v},
+    }
+    if "max_abs_err_vs_oracle" in rec:
+        line["max_abs_err_vs_oracle"] = error_summary(rec["max_abs_err_vs_oracle"])
+    for key in ("separation", "cpu_baseline"):
+        if key in rec:
+            line[key] = rec[key]
+    for name, r in subs.items():
+        c = {k: r[k] for k in ("workload", "value", "ms_per_step", "steps")}
+        c["e2e"] = {k: r["e2e"][k] for k in ("value", "ms_per_step", "d2h_bytes_per_step")}
+        c["kernels"] = kernel_summary(r["kernels"])
+        if "max_abs_err_vs_oracle" in r:
+            c["max_abs_err"] = r["max_abs_err_vs_oracle"]["max_abs"]
+            c["within_tol"] = r["max_abs_err_vs_oracle"]["within_tol"]
+        if "compare" in r:
+            m = r["compare"]["mixed"]
+            c["mixed"] = {k: m[k] for k in ("value", "ms_per_step", "all_certified")}
+        if "cpu_baseline" in r:
+            c["cpu_roots_per_s"] = r["cpu_baseline"]["value"]
+        line.setdefault("configs", {})[name] = c
+    if "compare" in rec:
+        m = rec["compare"]["mixed"]
+        line["mixed"] = {k: m[k] for k in ("value", "ms_per_step", "all_certified", "speedup_vs_fp64")}
+    return sig(line)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -816,6 +875,8 @@ def main():
     ap.add_argument("--sub", default=None, help="comma-separated configs reported beside the main one "
                                                 "(default with the default config: %s)" % DEFAULT_SUB)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
+    ap.add_argument("--record", default=None, help="file for the full record (per-step times, every kernel's "
+                                                   "figures); the printed line holds a summary of it")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-compare", action="store_true", help="skip the mixed-tier comparison and separation")
     args = ap.parse_args()
@@ -849,23 +910,10 @@ def main():
     for name in [x for x in sub.split(",") if x and x != args.config]:
         subs[name] = measure(b, name, min(args.steps, 10), 3, pk, peak_source, world, rank, with_cpu,
                              not args.no_compare, False)
-    kind, l, n, prec = cfg
-    line = {
-        "metric": METRIC, "value": main_rec["value"], "unit": "roots/s", "n_gpus": world, "steps": args.steps,
-        "warmup": args.warmup, "ms_per_step": main_rec["ms_per_step"], "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic (inputs fixed by n)",
-        "config": {"workload": main_rec["workload"], "precision": prec,
-                   "l2": "flushed between timed steps (256 MB write)",
-                   "parallelism": "replicas" if world > 1 else "single GPU"},
-        "e2e": main_rec["e2e"], "roofline": main_rec["roofline"], "kernels": main_rec["kernels"],
-        "peaks": {"fp64_tflops": pk["fp64"], "fp32_tflops": pk["fp32"], "source": peak_source},
-        "gpu_launches": main_rec["gpu_launches"], "clocks": main_rec["clocks"], "detail": main_rec["detail"],
-    }
-    for key in ("max_abs_err_vs_oracle", "compare", "separation", "cpu_baseline"):
-        if key in main_rec:
-            line[key] = main_rec[key]
-    if subs:
-        line["configs"] = subs
+    line = line_of(main_rec, subs, args.steps, args.warmup, world, pk)
+    if rank == 0 and args.record:
+        with open(args.record, "w") as f:
+            json.dump({"main": main_rec, "configs": subs}, f)
     if rank == 0:
         print(json.dumps(line), flush=True)
     if _POOL is not None:

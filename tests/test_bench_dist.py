@@ -177,3 +177,35 @@ def test_error_vs_oracle_on_the_host():
     zl[5] = 1e-17  # a double-double root: checked with its low part, against the dd tolerance
     e = bench.error_vs_oracle("hyp", 0, 10, z, zl, sample=64)
     assert e["checked_dd"] == 1 and e["checked_fp64"] >= 64 and e["max_abs_dd_roots"] > 5e-18
+
+
+def test_the_line_stays_short():
+    """The printed line with every part it can have and numbers of full length:
+    short enough that a reader of the last 8 KB of the output gets it whole."""
+    import json
+    import math
+    import bench
+    x = math.pi * 1e8
+    kern = [dict(bench._kernel("k_descend_mixed_%d" % i, "fp32", x, x, 3, x, x, "a description " * 8), traffic=x,
+                 traffic_unit="bytes per launch " * 4) for i in range(5)]
+    err = {k: x for k in ("max_abs", "max_abs_fp64_roots", "max_abs_dd_roots", "tol_fp64", "tol_dd", "checked_fp64",
+                          "checked_dd", "roots", "polish_last_step_max", "host_s")}
+    err.update(within_tol=True, how="binary128 " * 40)
+    rec = {"config_name": "c", "workload": "p_28 hyperbolic centres, " * 5, "value": x, "unit": "roots/s",
+           "ms_per_step": x, "steps": 20, "precision": "dd",
+           "e2e": {"value": x, "unit": "roots/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 4294968320,
+                   "ms_per_step": x, "call_ms": [x] * 500, "copy_ms": [x] * 500, "note": "n" * 320},
+           "roofline": bench.roofline_of(kern, "measured in this run " * 8), "kernels": kern, "gpu_launches": 100000,
+           "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 100},
+           "detail": {"ms_k_something_%d" % i: x for i in range(24)}, "max_abs_err_vs_oracle": err,
+           "compare": {"mixed": {"value": x, "ms_per_step": x, "all_certified": True, "speedup_vs_fp64": x, "kernels": kern}},
+           "cpu_baseline": {"value": x, "unit": "roots/s", "cores": 16, "kind": "oracle", "sample": "s" * 300},
+           "separation": {"ms": x, "set": "Hyp(28)", "roots": 1 << 27, "roots_per_s": x, "min_dist": x, "law": 118.4}}
+    line = bench.line_of(rec, {n: rec for n in bench.DEFAULT_SUB.split(",")}, 20, 5, 1,
+                         {"fp64": x, "fp32": x})
+    text = json.dumps(line)
+    assert len(text) < 8000, len(text)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"):
+        assert key in line, key
+    assert abs(line["value"] / x - 1) < 1e-5 and set(line["configs"]) == set(bench.DEFAULT_SUB.split(","))
