@@ -72,10 +72,11 @@ TOL_DD = 1e-20
 # arithmetic for an orbit of length m:
 #  - binary64 orbit with the scaled derivative: 6 FMA + 1 mul + 1 add per
 #    step, counted 13; the quotient with its range guard, the target or the
-#    update and the stop test 24.  k_descend, k_walk and k_descend_batch run
-#    this orbit in 64-bit fixed point on the integer pipes: their rate is
-#    given against the binary64 rate that it takes the place of, and may
-#    exceed it;
+#    update and the stop test 24;
+#  - the same orbit in 64-bit fixed point (k_descend, k_walk, k_descend_batch,
+#    except for the polynomials that fixed_point() leaves out): 19 integer
+#    multiply-adds a step, 12 of P' (cross terms 4 + 4, high products 2 + 2)
+#    and 7 of P; the value alone (the finish of p_23 to p_25) 7.  The quotient runs in binary32 beside them;
 #  - binary32 perturbation orbit (mixed tier): 19 flops per step in 12
 #    instructions (two FMA pairs for e, one FMA pair and an FMA/mul for g,
 #    four adds); the binary32 quotient, update and tests 25;
@@ -121,7 +122,15 @@ def finish_flops_fp64(m: int) -> int:
     return 7 * m + 2  # the orbit's value and z - q; the quotient and the tests run in binary32
 
 
-MIX_BATCH = 1 << 23  # starts per k_descend_mixed launch the line's per-launch figures refer to
+FIN_FIXED = (23, 25)  # orders of p_n whose finish has its value in fixed point
+IMADS, IMADS_VALUE = 19, 7  # integer multiply-adds of a fixed-point orbit step: P and P', P alone
+MIX_BATCH = 1 << 23  # starts per k_descend_mixed launch, for statistics without a count of timed launches
+
+
+def fixed_point(kind: str, l: int, n: int) -> bool:
+    """Whether the binary64 tier's walk and descents of a polynomial run in
+    fixed point (fixed_point_poly of the library; q_{l,n}: the walk only)."""
+    return not (n % 2 == 0 and ((kind == "mis" and l == 2) or (kind == "q" and l >= 2)))
 
 
 def nominal_peak(pipe: str, sm_mhz: float | None) -> float | None:
@@ -160,9 +169,22 @@ TRAFFIC = {
 }
 
 
+def in_fixed_point(k: dict, imads: float, peak: float | None) -> dict:
+    """A kernel's record against the integer multiply-adds that it runs on, where
+    their rate was measured; fp64_equiv: its binary64 count over the binary64 rate
+    in whose place it runs (above 1: faster than that pipe could be)."""
+    if not peak:
+        return k
+    s = k["ms_per_launch"] * k["launches"] / 1e3
+    a = imads / s / 1e12 if s > 0 else 0.0
+    k.update(fp64_equiv=k["frac"], pipe="imad", achieved=a, peak=peak, unit="1e12 multiply-adds/s", frac=a / peak,
+             frac_of_nominal=None)
+    return k
+
+
 def kernel_rooflines(kind: str, l: int, n: int, stats: list, pk: dict, sm_mhz: float | None = None) -> list:
-    """ALU roofline of each timed hot kernel against the FMA rate of its own
-    pipe: algorithmic flops (the kernels' own step counters x flops per step)
+    """ALU roofline of each timed hot kernel against the rate of its own
+    pipe (FMA, or integer multiply-add where that rate was measured): algorithmic flops (the kernels' own step counters x flops per step)
     over the kernel's device time (CUDA events around its launches on the
     launch stream, inside the CUDA graph), mean over the timed steps."""
     s0 = stats[-1]
@@ -172,43 +194,51 @@ def kernel_rooflines(kind: str, l: int, n: int, stats: list, pk: dict, sm_mhz: f
         return statistics.mean(float(s[key]) for s in stats)
 
     out = []
-    p64, p32 = pk.get("fp64"), pk.get("fp32")
+    p64, p32, imad = pk.get("fp64"), pk.get("fp32"), pk.get("imad")
     n64, n32 = nominal_peak("fp64", sm_mhz), nominal_peak("fp32", sm_mhz)
+    mixed = s0.get("desc_fp32", 0) > 0
+    long = kind == "hyp" and m >= LONG_MIN
+    fx = fixed_point(kind, l, n)
     if s0.get("ms_k_desc64", 0) > 0 and s0.get("desc_orbit_steps", 0) > 0:  # the batched split
         steps, orb = s0["desc_newton"], s0["desc_orbit_steps"]
-        out.append(_kernel("k_descend_batch", "fp64", 13 * orb + 24 * steps, mean("ms_k_desc64"), 1, p64, n64,
-                           "Newton steps %d in fixed point (integer pipes, against the binary64 rate): 13 flops x %d orbit steps + 24 x steps" % (steps, orb)))
+        k = _kernel("k_descend_batch", "fp64", 13 * orb + 24 * steps, mean("ms_k_desc64"), 1, p64, n64,
+                    "Newton steps %d: 13 flops x %d orbit steps + 24 x steps (fixed point but for s_{2,n}, n even)" % (steps, orb))
+        out.append(in_fixed_point(k, IMADS * orb, imad))
     elif s0.get("ms_k_desc64", 0) > 0:
         per = 13 * n + 50 * l + 24 if kind == "q" else newton_flops(m)
         # in the mixed tier desc_newton also counts the binary32 steps and the
         # binary64 finish; the binary64 descent kernel ran the tip redo only
+        # (of short orbits in binary64)
         steps = s0["desc_newton"] - s0.get("desc_fp32", 0) - s0.get("finish_newton", 0)
-        out.append(_kernel("k_descend_q" if kind == "q" else "k_descend", "fp64", steps * per, mean("ms_k_desc64"),
-                           1, p64, n64, "%s Newton steps %d x %d flops" %
-                           ("binary64" if kind == "q" else "fixed-point (integer pipes, against the binary64 rate)", steps, per)))
+        fixed = fx and kind != "q" and not (mixed and kind == "hyp" and not long)
+        k = _kernel("k_descend_q" if kind == "q" else "k_descend", "fp64", steps * per, mean("ms_k_desc64"), 1, p64, n64,
+                    "%s Newton steps %d x %d flops" % ("fixed-point" if fixed else "binary64", steps, per))
+        out.append(in_fixed_point(k, IMADS * m * steps, imad) if fixed else k)
     if s0.get("ms_k_desc32", 0) > 0:
         steps = s0["desc_fp32"]
-        launches = -(-s0["n_starts"] // MIX_BATCH)
-        if kind == "hyp" and m >= LONG_MIN:
-            launches = 2  # all starts, then the far list
+        # the library times the walk, these launches (from p_23 on a second one,
+        # the far list), the finish and the tip redo
+        launches = max(1, s0["n_k_timed"] - 3) if "n_k_timed" in s0 else -(-s0["n_starts"] // MIX_BATCH)
         flops, work = descent_flops_fp32(kind, m, steps, s0["n_starts"])
         out.append(_kernel("k_descend_mixed", "fp32", flops, mean("ms_k_desc32"), launches, p32, n32, work))
     if s0.get("ms_k_finish", 0) > 0:
         steps = s0["finish_newton"]
-        out.append(_kernel("k_finish_f64", "fp64", steps * finish_flops_fp64(m), mean("ms_k_finish"), 1, p64, n64,
-                           "binary64 finish steps %d x %d flops" % (steps, finish_flops_fp64(m))))
+        fixed = kind == "hyp" and FIN_FIXED[0] <= m <= FIN_FIXED[1]
+        k = _kernel("k_finish_f64", "fp64", steps * finish_flops_fp64(m), mean("ms_k_finish"), 1, p64, n64,
+                    "%s finish steps %d x %d flops" % ("fixed-point" if fixed else "binary64", steps, finish_flops_fp64(m)))
+        out.append(in_fixed_point(k, IMADS_VALUE * m * steps, imad) if fixed else k)
     if s0.get("ms_k_walk", 0) > 0:
         steps = s0["walk_newton"] - s0["seed_newton"]
         if s0["steps_fp32"] > 0:  # binary32 walk sub-steps (the binary64 anchors are not counted)
-            long = kind == "hyp" and m >= LONG_MIN  # the series' length varies by turn
+            # the series' length varies by turn
             out.append(_kernel("k_walk_series" if long else "k_walk_mixed", "fp32", steps * newton_flops_fp32(m),
                                mean("ms_k_walk"), 1, p32, n32, "binary32 walk steps %d x %d flops (anchors not "
                                "counted%s)" % (steps, newton_flops_fp32(m), "; whole orbits, although a series "
                                                "takes the place of their first steps" if long else "")))
         else:
-            out.append(_kernel("k_walk", "fp64", steps * newton_flops(m), mean("ms_k_walk"), 1, p64, n64,
-                               "fixed-point walk steps (integer pipes, against the binary64 rate) %d x %d flops" % (steps, newton_flops(m))))
-    mixed = s0.get("desc_fp32", 0) > 0
+            k = _kernel("k_walk", "fp64", steps * newton_flops(m), mean("ms_k_walk"), 1, p64, n64,
+                        "%s walk steps %d x %d flops" % ("fixed-point" if fx else "binary64", steps, newton_flops(m)))
+            out.append(in_fixed_point(k, IMADS * m * steps, imad) if fx else k)
     for k in out:  # DRAM bytes per launch: measured bytes per unit x this launch's units
         t = TRAFFIC.get(k["kernel"])
         if t is None or (k["kernel"] == "k_descend" and mixed) or kind != "hyp":
@@ -777,7 +807,7 @@ def measure(b: Bench, name: str, steps: int, warmup: int, pk: dict, peak_source:
         "detail": {k: s0.get(k) for k in (
             "ms_walk", "ms_seeds", "ms_descend", "ms_dedup", "ms_certify", "ms_dd", "ms_k_walk", "ms_k_desc64",
             "ms_k_desc32", "ms_k_finish", "walk_newton", "seed_newton", "desc_newton", "desc_fp32",
-            "finish_newton", "n_finish", "n_chunks", "n_zones", "n_zone_roots", "steps_dd", "prec_used")},
+            "finish_newton", "n_finish", "n_k_timed", "n_chunks", "n_zones", "n_zone_roots", "steps_dd", "prec_used")},
     }
     rec["detail"]["wall_s"] = wall
     if rank == 0 and world == 1 and kind != "q":
@@ -816,7 +846,7 @@ def sig(x, digits: int = 6):
 
 
 def kernel_summary(kernels: list) -> list:
-    return [{k: x[k] for k in ("kernel", "pipe", "frac", "ms_per_launch", "launches")} for x in kernels]
+    return [{k: x[k] for k in ("kernel", "pipe", "frac", "fp64_equiv", "ms_per_launch", "launches") if k in x} for x in kernels]
 
 
 def error_summary(e: dict) -> dict:
@@ -839,7 +869,7 @@ def line_of(rec: dict, subs: dict, steps: int, warmup: int, world: int, pk: dict
                    "parallelism": "replicas" if world > 1 else "single GPU"},
         "e2e": {k: rec["e2e"][k] for k in keep}, "gpu_launches": rec["gpu_launches"], "clocks": rec["clocks"],
         "roofline": rec["roofline"], "kernels": kernel_summary(rec["kernels"]),
-        "peaks": {"fp64_tflops": pk["fp64"], "fp32_tflops": pk["fp32"]},
+        "peaks": {"fp64_tflops": pk["fp64"], "fp32_tflops": pk["fp32"], "imad_t_per_s": pk.get("imad")},
         "detail": {k: v for k, v in rec["detail"].items() if v},
     }
     if "max_abs_err_vs_oracle" in rec:
@@ -898,9 +928,9 @@ def main():
     stream = torch.cuda.Stream()
     torch.cuda.set_stream(stream)
     # FMA rates of this GPU, measured here (the ALU rooflines' denominators)
-    pk = {"fp64": mt.fma_peak("fp64"), "fp32": mt.fma_peak("fp32")}
-    peak_source = ("measured in this run by mt_fma_peak (independent FMA chains on every SM, CUDA events): "
-                   "binary64 %.3f, binary32 %.1f TFLOP/s" % (pk["fp64"], pk["fp32"]))
+    pk = {"fp64": mt.fma_peak("fp64"), "fp32": mt.fma_peak("fp32"), "imad": mt.imad_peak()}
+    peak_source = ("measured in this run by mt_fma_peak, mt_imad_peak (independent chains on every SM, CUDA events): "
+                   "binary64 %.3f, binary32 %.1f TFLOP/s, integer multiply-add %.2f T/s" % (pk["fp64"], pk["fp32"], pk["imad"]))
     b = Bench(mt, torch, stream, dist)
     with_cpu = not args.no_cpu_baseline
     main_rec = measure(b, args.config, args.steps, args.warmup, pk, peak_source, world, rank, with_cpu,

@@ -395,6 +395,11 @@ MT_API mt_status mt_certify_static(int kind, int l, int n, const double* d_roots
 MT_API size_t mt_fma_peak_workspace_bytes(void);
 MT_API mt_status mt_fma_peak(int prec, void* d_work, size_t work_bytes, double* tflops, void* stream);
 
+/* The same for the 32 x 32 + 64 bit integer multiply-add, which bounds the
+   fixed-point orbits of the binary64 tier, in 10^12 multiply-adds a second
+   (d_work as for mt_fma_peak). */
+MT_API mt_status mt_imad_peak(void* d_work, size_t work_bytes, double* tops, void* stream);
+
 /* Self-check of the certificate's binary32 square-root upper bound (Thm
    proofRoots needs upper bounds of |z| and |p'|; the disk orbit takes them
    as sqrt.approx.f32 times 1 + 2^-19, rounded upward): over every normal

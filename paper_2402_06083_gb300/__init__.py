@@ -366,6 +366,17 @@ def fma_peak(prec: str = "fp64") -> float:
     return float(out.value)
 
 
+def imad_peak() -> float:
+    """Rate of the 32 x 32 + 64 bit integer multiply-add of the current GPU, in
+    10^12 a second (mt_imad_peak): the bound of the fixed-point orbits."""
+    torch = _torch()
+    L = load()
+    buf = torch.empty(int(L.mt_fma_peak_workspace_bytes()), dtype=torch.uint8, device="cuda")
+    out = ctypes.c_double(0.0)
+    check(L.mt_imad_peak(buf.data_ptr(), buf.numel(), ctypes.byref(out), torch.cuda.current_stream().cuda_stream))
+    return float(out.value)
+
+
 def check_sqrt_up() -> tuple:
     """mt_check_sqrt_up: (failures, largest relative error) of the
     certificate's binary32 square-root upper bound over every normal

@@ -209,3 +209,32 @@ def test_the_line_stays_short():
                 "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"):
         assert key in line, key
     assert abs(line["value"] / x - 1) < 1e-5 and set(line["configs"]) == set(bench.DEFAULT_SUB.split(","))
+
+
+def test_rooflines_name_the_pipe_that_runs():
+    """With the integer rate measured, fixed-point kernels are held against it,
+    19 multiply-adds an orbit step (7 for the finish's value), and the
+    polynomials kept in binary64 against binary64; launches as timed."""
+    import bench
+    pk = {"fp64": 1.25, "fp32": 78.0, "imad": 9.0}
+    by = lambda *a: {k["kernel"]: k for k in bench.kernel_rooflines(*a, pk)}
+    k = by("hyp", 0, 20, [_stats()])
+    assert k["k_descend"]["pipe"] == "imad" and abs(k["k_descend"]["frac"] - 19 * 20 * 2000 / 3e-3 / 9e12) < 1e-12
+    assert abs(k["k_descend"]["fp64_equiv"] - 2000 * (13 * 20 + 24) / 3e-3 / 1.25e12) < 1e-12
+    assert k["k_walk"]["pipe"] == "imad"
+    k = by("mis", 2, 14, [_stats()])  # roots 0, +-i: binary64
+    assert k["k_descend"]["pipe"] == k["k_walk"]["pipe"] == "fp64" and "binary64" in k["k_walk"]["work"]
+    k = by("q", 9, 8, [_stats()])
+    assert k["k_descend_q"]["pipe"] == k["k_walk"]["pipe"] == "fp64"
+    k = by("q", 9, 9, [_stats()])
+    assert k["k_descend_q"]["pipe"] == "fp64" and k["k_walk"]["pipe"] == "imad"
+    assert bench.kernel_rooflines("mis", 0, 15, [_stats(desc_orbit_steps=30000)], pk)[0]["pipe"] == "imad"
+    st = dict(desc_fp32=1500, steps_fp32=1600, finish_newton=400, ms_k_desc32=1.0, ms_k_finish=2.5, n_finish=300,
+              n_starts=(1 << 24) + 1)
+    k = by("hyp", 0, 24, [_stats(n_k_timed=5, **st)])
+    assert k["k_descend_mixed"]["launches"] == 2 and k["k_finish_f64"]["pipe"] == "imad"
+    assert abs(k["k_finish_f64"]["achieved"] - 7 * 24 * 400 / 2.5e-3 / 1e12) < 1e-12
+    k = by("hyp", 0, 22, [_stats(n_k_timed=4, **st)])
+    assert k["k_descend_mixed"]["launches"] == 1 and k["k_finish_f64"]["pipe"] == "fp64"
+    assert k["k_descend"]["pipe"] == "fp64"  # the tip redo of a short orbit
+    assert by("mis", 8, 10, [_stats(n_k_timed=4, **st)])["k_descend_mixed"]["launches"] == 1
