@@ -683,9 +683,9 @@ mt_status enqueue_pass(const Plan& p, const Buffers& b, double2* out, double2* o
     // end points in keys / vals, the finish lists in flag / pos / vals_alt / type
     FinishScratch fin{b.keys, b.keys_alt, b.vals, b.vals_alt, b.flag, b.pos, b.vals_alt, b.type,
                       b.scan_tmp, b.radix_tmp, &b.ctr->n_finish};
-    CK(launch_descend_mixed(p.P, b.starts, p.S, p.tol, p.cap, b.cand, b.status, b.anchors, fin, b.ctr, s));
+    CK(launch_descend_mixed(p.P, b.starts, p.S, p.tol, p.cap, p.eps, b.cand, b.status, b.anchors, fin, b.ctr, s));
   } else {
-    CK(launch_descend(p.P, b.starts, p.S, p.tol, p.cap, b.cand, b.status, b.ctr, 0, s));
+    CK(launch_descend(p.P, b.starts, p.S, p.tol, p.cap, p.eps, b.cand, b.status, b.ctr, 0, s));
   }
   CK(mark(ev.e[2], s, capturing));
   if (p.prec == MT_MIXED) {
@@ -785,9 +785,9 @@ mt_status run_streamed(const Plan& p, const Buffers& b, double2* out, double2* o
       // end points in keys / vals, the finish lists in flag / pos / vals_alt / type
       FinishScratch fin{b.keys, b.keys_alt, b.vals, b.vals_alt, b.flag, b.pos, b.vals_alt, b.type,
                         b.scan_tmp, b.radix_tmp, &b.ctr->n_finish};
-      CK(launch_descend_mixed(p.P, b.starts, Sk, p.tol, p.cap, b.cand, b.status, b.anchors, fin, b.ctr, s));
+      CK(launch_descend_mixed(p.P, b.starts, Sk, p.tol, p.cap, p.eps, b.cand, b.status, b.anchors, fin, b.ctr, s));
     } else {
-      CK(launch_descend(p.P, b.starts, Sk, p.tol, p.cap, b.cand, b.status, b.ctr, 0, s));
+      CK(launch_descend(p.P, b.starts, Sk, p.tol, p.cap, p.eps, b.cand, b.status, b.ctr, 0, s));
     }
     CK(cudaEventRecord(pe[4 * k + 2], s));
     CK(launch_piece_valid(b.ctr, snap, nvalid, s));
@@ -1375,7 +1375,7 @@ mt_status run_batch_pass(const BatchPlan& b, const BatchBuffers& r, double2* out
   CK(launch_walk_batch(r.E, r.chunk_off, b.np, b.chunks_total, b.lambda0, b.M, b.every, r.seeds,
                        r.starts, r.ctr, s));
   CK(cudaEventRecord(ev.e[1], s));
-  CK(launch_descend_batch(r.E, r.start_off, b.np, b.S, b.tol, r.starts, r.cand, r.status, r.seg,
+  CK(launch_descend_batch(r.E, r.start_off, b.np, b.S, b.tol, b.eps, r.starts, r.cand, r.status, r.seg,
                           r.ctr, s));
   CK(cudaEventRecord(ev.e[2], s));
   SegView sv;
@@ -2013,7 +2013,7 @@ mt_status mt_descend(int kind, int l, int n, const mt_options* opts, const doubl
   cudaStream_t s = (cudaStream_t)o->stream;
   DevCounters* ctr = (DevCounters*)d_work;
   CK(launch_init_counters(ctr, s));
-  CK(launch_descend(p.P, (const double2*)d_starts, count, p.tol, p.cap, (double2*)d_out, d_status,
+  CK(launch_descend(p.P, (const double2*)d_starts, count, p.tol, p.cap, 0.0, (double2*)d_out, d_status,
                     ctr, o->block, s));
   DevCounters h;
   CK(cudaMemcpyAsync(&h, ctr, sizeof(h), cudaMemcpyDeviceToHost, s));

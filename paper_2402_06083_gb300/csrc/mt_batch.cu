@@ -66,11 +66,26 @@ __global__ void k_walk_batch(const BatchEntry* __restrict__ E, const int64_t* __
   warp_add_u64(&ctr->walk_fail, fails);
 }
 
+// axis_add (mt_newton.cu) with the polynomial of each entry
+static __device__ __noinline__ unsigned axis_add_batch(const BatchEntry* E, const uint16_t* seg, int64_t* buf,
+                                                       unsigned n, bool mine, int64_t at, double2* cand,
+                                                       unsigned flush) {
+  axis_push(buf, n, mine, at);
+  if (n >= flush) {
+    int64_t i;
+    if (axis_pop(buf, n, i)) {
+      const PolyDev& P = E[seg[i]].P;
+      cand[i] = axis_step(P.m, P.lcap, cand[i]);
+    }
+  }
+  return n;
+}
+
 // persistent Newton descents over the starts of all polynomials (k_descend
 // with the polynomial looked up per start)
 __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restrict__ E,
                                                        const int64_t* __restrict__ start_off,
-                                                       int np, int64_t count, float tol2,
+                                                       int np, int64_t count, float tol2, unsigned axis_lo,
                                                        const double2* __restrict__ starts,
                                                        double2* __restrict__ cand,
                                                        uint8_t* __restrict__ status,
@@ -85,13 +100,6 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
   __shared__ int64_t axis_buf[4][64];
   int64_t* abuf = axis_buf[threadIdx.x >> 5];
   unsigned na = 0;
-  auto axis = [&]() {
-    int64_t i;
-    if (axis_pop(abuf, na, i)) {
-      const PolyDev& P = E[seg[i]].P;
-      cand[i] = axis_step(P.m, P.lcap, cand[i]);
-    }
-  };
   for (;;) {
     // as k_descend: written and refilled together once DESC_REFILL lanes wait
     const unsigned running = __ballot_sync(0xffffffffu, idx >= 0 && idx < count && outcome < 0);
@@ -102,7 +110,7 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
       if (outcome >= 0) {
         const double2 z = descent_point(d);
         cand[at] = z;
-        near = outcome == 0 && d.fx && fx_below(z.y, AXIS_EXP);
+        near = outcome == 0 && d.fx && axis_near(z, axis_lo);
         status[at] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
@@ -110,8 +118,7 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
         outcome = -1;
         idx = -1;
       }
-      axis_push(abuf, na, near, at);
-      if (na >= 32u) axis();
+      if (__any_sync(0xffffffffu, near)) na = axis_add_batch(E, seg, abuf, na, near, at, cand, 32u);
       const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
       if (need) {
         unsigned long long base = 0;
@@ -145,7 +152,7 @@ __global__ void __launch_bounds__(128) k_descend_batch(const BatchEntry* __restr
       orbit += (unsigned)m;
     }
   }
-  if (na) axis();
+  if (na) axis_add_batch(E, seg, abuf, na, false, 0, cand, 1u);
   warp_add_u64(&ctr->desc_newton, steps);
   warp_add_u64(&ctr->desc_orbit, orbit);
   warp_add_u64(&ctr->n_conv, nconv);
@@ -181,7 +188,7 @@ cudaError_t launch_walk_batch(const BatchEntry* E, const int64_t* chunk_off, int
   if (total <= 0) return cudaSuccess;
   const int bs = 64;
   int per_sm = 0;
-  const int fb = lambda0 <= 12.0 ? 28 : lambda0 <= 200.0 ? 26 : 0;  // as walk_fb
+  const int fb = level_fb(lambda0);  // (walk_chunk_from reads each polynomial's fx)
   const auto kern = fb == 28 ? &k_walk_batch<28> : fb == 26 ? &k_walk_batch<26> : &k_walk_batch<0>;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, bs, 0);
   if (e != cudaSuccess) return e;
@@ -195,7 +202,7 @@ cudaError_t launch_walk_batch(const BatchEntry* E, const int64_t* chunk_off, int
 }
 
 cudaError_t launch_descend_batch(const BatchEntry* E, const int64_t* start_off, int np,
-                                 int64_t count, double tol, const double2* starts, double2* cand,
+                                 int64_t count, double tol, double eps, const double2* starts, double2* cand,
                                  uint8_t* status, uint16_t* seg, DevCounters* ctr, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   const int bs = 128;
@@ -206,7 +213,7 @@ cudaError_t launch_descend_batch(const BatchEntry* E, const int64_t* start_off, 
   const int64_t need = (count + bs - 1) / bs;
   if (grid > need) grid = need;
   MT_COUNT_LAUNCH(1);
-  k_descend_batch<<<(unsigned)grid, bs, 0, s>>>(E, start_off, np, count, tol2_f(tol), starts, cand,
+  k_descend_batch<<<(unsigned)grid, bs, 0, s>>>(E, start_off, np, count, tol2_f(tol), axis_floor(eps), starts, cand,
                                                 status, seg, ctr);
   return cudaGetLastError();
 }

@@ -9,7 +9,8 @@
 // 15); a dependent binary64 operation waits 64 clocks, an integer one 4 to 10.
 // No step needs a wide exponent range: on and inside the level line |p_k|
 // stays below sqrt(lambda0 + 3), and outside it the descent is still far from
-// every root.  Bound: the integer multiply-add pipe.  Tried and not kept: the
+// every root.  Bound: issue and the integer pipes (k_descend at p_20: 63 % issue,
+// 50 % ALU pipe, half of the measured multiply-add rate).  Tried and not kept: the
 // derivative in float-float (37 clocks, packed pairs 35), its cross terms in
 // binary32 (37), a normalisation every step (39).  Split of p_20: descents
 // 2.70 -> 0.84 ms, walk 2.32 -> 0.62, seeds 0.60 -> 0.33.
@@ -17,8 +18,7 @@
 // Numbers.  A coordinate is an integer X of 64 bits, value X 2^-(FB+32), held
 // as two signed limbs h 2^32 + l: FB bits of fraction in the high limb, the
 // components below 2^(30 - FB) (FB = 28: 4, FB = 26: 16) by one unit of the
-// high limb or more.  A product keeps
-// 2 FB fractional bits: h h exactly plus the cross terms h l + l h, rounded
+// high limb or more.  A product keeps 2 FB fractional bits: h h exactly plus the cross terms h l + l h, rounded
 // to nearest (the l l term, below a quarter of the last place, is dropped),
 // so a step z^2 + c is off by at most 3/4 2^-2FB in each component: 1.04e-17
 // for FB = 28, where two binary64 roundings of values in [1, 2) are 2.2e-16.
@@ -28,9 +28,12 @@
 // Near a root the quotient P / P' is off by 3.5e-18 rms for FB = 28 (1e-17 for
 // 27, 4e-17 for 26), in binary64 by 3.5e-17 (against binary128, p_5 to p_32
 // and s_{l,n} to order 25).
+// The errors are absolute: a component below 1e-4 is less exact than in binary64,
+// whose error shrinks with it, and the descents take it from there (axis_step,
+// mt_descent.cuh).
 // Orbits that leave the fixed range before their last step go on in
-// float-float (they are far from every root: |p_k| > 2 escapes), and what
-// leaves binary32's range is left to the caller's binary64 path.
+// float-float (they are far from every root: |p_k| > 2 escapes), from |p_k|^2 =
+// 2^60 on by halving P / P'; one past binary64's range is reported.
 #pragma once
 #include <cstdint>
 

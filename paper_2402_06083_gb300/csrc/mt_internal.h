@@ -106,16 +106,17 @@ cudaError_t launch_walk(const PolyDev& P, double lambda0, int M, int every, int6
                         int64_t nchunks, const double2* seeds, double2* starts, DevCounters* ctr,
                         cudaStream_t s, int block = 64);
 
-// a4: persistent Newton descent over 'count' starts.
+// a4: persistent Newton descent over 'count' starts.  eps: the caller folds
+// |Im| < eps / 2 to the real axis afterwards (0: it does not).
 cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t count, double tol,
-                           int cap, double2* cand, uint8_t* status, DevCounters* ctr, int block,
+                           int cap, double eps, double2* cand, uint8_t* status, DevCounters* ctr, int block,
                            cudaStream_t s);
 // The same descents (binary64, stop rules of launch_descend) from the
 // starts list[0 .. *nlist) only; outcomes at the listed indices, not
 // counted in ctr (the caller counts them).
 cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const uint32_t* list,
                                 const unsigned long long* nlist, int64_t count, double tol, int cap,
-                                double2* cand, uint8_t* status, DevCounters* ctr, cudaStream_t s);
+                                double eps, double2* cand, uint8_t* status, DevCounters* ctr, cudaStream_t s);
 
 // a1-a4 in the mixed tier (binary32 perturbation around binary64 anchors).
 // seed_bad [N0/2 + 1] and chunk_fail [nchunks] receive the per-item
@@ -149,7 +150,7 @@ struct FinishScratch {
 // starts: in, the starts; out, the binary32 end points (binary64 values,
 // folded into the upper half where a finish followed).  cand: the
 // candidates (also the binary32 deltas and scales before the finish).
-cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t count, double tol, int cap,
+cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t count, double tol, int cap, double eps,
                                  double2* cand, uint8_t* status, void* anchors, const FinishScratch& fin,
                                  DevCounters* ctr, cudaStream_t s);
 size_t mixed_anchor_bytes(const PolyDev& P, int64_t count);
@@ -162,7 +163,7 @@ cudaError_t launch_walk_batch(const BatchEntry* E, const int64_t* chunk_off, int
                               double lambda0, int M, int every, const double2* seeds,
                               double2* starts, DevCounters* ctr, cudaStream_t s);
 cudaError_t launch_descend_batch(const BatchEntry* E, const int64_t* start_off, int np,
-                                 int64_t count, double tol, const double2* starts, double2* cand,
+                                 int64_t count, double tol, double eps, const double2* starts, double2* cand,
                                  uint8_t* status, uint16_t* seg, DevCounters* ctr, cudaStream_t s);
 cudaError_t launch_seg_keys(const uint32_t* vals, const uint16_t* seg, const uint8_t* status,
                             int64_t count, uint64_t* keys, cudaStream_t s);

@@ -345,11 +345,10 @@ __device__ __forceinline__ bool walk_chunk_from(const PolyDev& P, double lambda0
 
 // The fraction bits for the walk of |P| = lambda0: the largest orbit value is
 // |p_{m-1}| <= sqrt(lambda0 + |c| + |p_lcap|), |c| < 2.3 on lines of degree 16
-// and more, which must stay below 2^(30 - FB): 28 up to lambda0 = 12, 26 up to
-// 200, binary64 (0) beyond.
-inline int walk_fb(const PolyDev& P, double lambda0) {
-  return !P.fx ? 0 : lambda0 <= 12.0 ? 28 : lambda0 <= 200.0 ? 26 : 0;
-}
+// and more, which is to stay below 2^(30 - FB) (past it the step is right, but
+// slower): 28 up to lambda0 = 12, 26 up to 200, binary64 (0) beyond.
+inline int level_fb(double lambda0) { return lambda0 <= 12.0 ? 28 : lambda0 <= 200.0 ? 26 : 0; }
+inline int walk_fb(const PolyDev& P, double lambda0) { return P.fx ? level_fb(lambda0) : 0; }
 
 // The phases of a turn, in binary64 and at 2^-2FB (block-wide).
 template <int FB>

@@ -1,6 +1,7 @@
 // mt_mixed.cu -- the mixed-precision tier (MT_MIXED): binary32 level-line
 // tracking and early Newton steps around float-float anchors (binary64 ones
-// in the seed lift), and a binary64 finish.
+// in the seed lift), and a finish with the value in 64 bits: binary64, or fixed
+// point (mt_fix.cuh) for p_23 to p_25.
 //
 // Why.  The paper runs everything in FP80 (Sec. 6.1) and notes that GPUs
 // offer little beyond FP64 (Sec. 6.4.5).  On a GB300 the binary64 pipe is
@@ -21,12 +22,12 @@
 // (Z_m - T) + e_m with Z_m split into binary32 hi + lo.
 //   - Walk: the anchor is re-taken every K sub-steps (a few turns of the
 //     phase) from the current point, so |delta| stays a few turns' length.
-//   - Descent: the anchor is the start point; binary32 Newton steps run to
-//     the binary32 floor, then binary64 Newton steps (1.08 a root at p_28),
-//     once per group of end points on the same root, finish to the binary64
-//     tolerance (eq. Newton).
+//   - Descent: the anchor is the start point (p_n from 23 on: one of four
+//     consecutive starts); binary32 Newton steps run to the binary32 floor, then
+//     64-bit Newton steps (1.08 a root at p_28), once per group of end points on
+//     the same root, finish to the tolerance (eq. Newton).
 // The anchors only steer the binary32 steps; every root's digits come from
-// its binary64 finishing steps.  The chunk-end check of the walk and the
+// its 64-bit finishing steps.  The chunk-end check of the walk and the
 // count check catch any tracking failure, and the host then repeats the
 // split in plain binary64.
 #include "mt_descent.cuh"
@@ -38,9 +39,10 @@ namespace mt {
 
 constexpr int MIX_MAXM = 41;
 // Shorter orbits of p_n keep an anchor per start, the whole orbit and the
-// binary64 finish and tip redo: the splits are short there (p_20: 5 % of 1.36
-// ms from all of them), and the last digits of their roots, on which the
-// nearest-neighbour distances at the tip rest, stay as they were.
+// binary64 finish and tip redo.  Not for their speed: all four of the long orbits'
+// ways take p_20 from 1.36 to 1.30 ms (the walk's series alone is slower there, see
+// WALK_SERIES_MIN).  The last digits of these roots are what nearest-neighbour
+// distances at the tip rest on, and they stay those of binary64.
 constexpr int MIX_LONG = 23;
 inline bool mixed_short(const PolyDev& P) { return P.kind == 0 && P.m < MIX_LONG; }
 // The binary64 finish in fixed point: p_23 to p_25.  Of p_28's 67 M roots some
@@ -523,10 +525,11 @@ WalkMixedFn walk_mixed_fixed(int m) {
     return m == MC ? &k_walk_mixed<false, MC> : walk_mixed_fixed<MC - 1>(m);
   }
 }
-// From p_23 on: below, the line's lanes are too few and the anchors' votes and
-// the loop over a varying length only add latency (ms of the walk, without and
-// with the series: p_20 0.178 and 0.212, p_21 0.222 and 0.246, p_22 0.408 and
-// 0.365, p_24 1.63 and 1.36, p_28 24.9 and 17.8).
+// ms of the walk, without and with the series: p_20 0.178 and 0.212, p_21 0.222
+// and 0.246 (the line's lanes are too few, and the anchors' votes and the loop over
+// a varying length add latency), p_22 0.408 and 0.365, p_24 1.63 and 1.50, p_28
+// 24.9 and 19.6.  By time the line lies between p_21 and p_22; p_22 stays with the
+// short orbits (MIX_LONG).
 constexpr int WALK_SERIES_MIN = MIX_LONG;
 WalkMixedFn walk_mixed_kernel(const PolyDev& P) {
   if (P.lcap >= 0) return &k_walk_mixed<true, 0>;
@@ -780,7 +783,9 @@ __global__ void __launch_bounds__(DM_BS) k_descend_mixed(PolyDev P, int Kr, int 
       d0x = d0y = 0.f;
     } else {
       const double2 s0 = starts[at], c0 = ws.c0[j];
-      d0x = f32_trunc(s0.x - c0.x);  // exact differences, zero for the anchor itself
+      // truncated to 2^-23 of the difference, the order of binary32's rounding of
+      // the steps' delta; zero for the anchor itself
+      d0x = f32_trunc(s0.x - c0.x);
       d0y = f32_trunc(s0.y - c0.y);
       dx = d0x;
       dy = d0y;
@@ -1114,14 +1119,14 @@ __global__ void k_finish_list(int64_t count, const uint32_t* __restrict__ head, 
 // binary64 (the polynomials kept there).  Bound: the integer multiply-add
 // pipe (56 %) and issue (70 %); in binary64 that pipe's 3 FMA a step, 16 clocks
 // a warp each, with the heads outside the line repeating six steps.  p_24, 4.5 M
-// heads: 0.865 -> 0.305 ms, 0.03 of it the binary64 step of the small imaginary
+// heads: 0.865 -> 0.282 ms, 0.01 of it the binary64 step of the small imaginary
 // parts (axis_step) (p_28 15.1 -> 4.65 without it; not taken there, FIN_FX_MAXM).
 constexpr int FIN_FB = 28;
 constexpr unsigned FIN_REFILL = 6;
 template <bool FX>
 __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* __restrict__ list,
                                                     const unsigned long long* __restrict__ nlist,
-                                                    int64_t cap_list, double tol2, int cap,
+                                                    int64_t cap_list, double tol2, int cap, unsigned axis_lo,
                                                     const double2* __restrict__ c32,
                                                     double2* __restrict__ cand,
                                                     uint8_t* __restrict__ status,
@@ -1152,7 +1157,7 @@ __global__ void __launch_bounds__(128) k_finish_f64(PolyDev P, const uint32_t* _
         if (FX) {
           zx = fx_to_f64<FIN_FB>(X);
           zy = fx_to_f64<FIN_FB>(Y);
-          near = outcome == 0 && fx_below(zy, AXIS_EXP);
+          near = outcome == 0 && axis_near(make_double2(zx, zy), axis_lo);
         }
         cand[at] = make_double2(zx, zy);
         status[at] = (uint8_t)outcome;
@@ -1370,7 +1375,7 @@ static cudaError_t launch_dm(DescMixedFn kern, const PolyDev& P, int K, int gsh,
   return ktimer_end(s);
 }
 
-cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t count, double tol, int cap,
+cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t count, double tol, int cap, double eps,
                                  double2* cand, uint8_t* status, void* anchors, const FinishScratch& fin,
                                  DevCounters* ctr, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
@@ -1439,7 +1444,8 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
     if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess) return e;
     MT_COUNT_LAUNCH(1);
     if ((e = ktimer_begin(KS_FINISH, s)) != cudaSuccess) return e;
-    kfin<<<(unsigned)fgrid, bs, 0, s>>>(P, fin.list, fin.nheads, count, tol * tol, 6, starts, cand, status, q, ctr);
+    kfin<<<(unsigned)fgrid, bs, 0, s>>>(P, fin.list, fin.nheads, count, tol * tol, 6, axis_floor(eps), starts, cand, status, q,
+                                     ctr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = ktimer_end(s)) != cudaSuccess) return e;
   }
@@ -1454,7 +1460,7 @@ cudaError_t launch_descend_mixed(const PolyDev& P, double2* starts, int64_t coun
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   PolyDev Pt = P;
   if (mixed_short(P)) Pt.fx = 0;
-  if ((e = launch_descend_list(Pt, starts, fin.pos, n2, count, tol, cap, cand, status, ctr, s)) != cudaSuccess)
+  if ((e = launch_descend_list(Pt, starts, fin.pos, n2, count, tol, cap, eps, cand, status, ctr, s)) != cudaSuccess)
     return e;
   MT_COUNT_LAUNCH(2);
   k_finish_append<<<sgrid, bs, 0, s>>>(fin.pos, n2, fin.list, fin.nheads, count, status, ctr);

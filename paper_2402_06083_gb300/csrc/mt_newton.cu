@@ -20,12 +20,27 @@
 
 namespace mt {
 
+// axis_push and the step of 32 entries in one call, out of line: in line it took
+// the loop's registers (p_12 0.3094 ms a split, 0.3076 so; 0.3065 without any
+// step).  A kernel of its own over all candidates is cheaper for long lists of
+// s_{l,n} (s_{4,22} 51.9 -> 50.5 ms, 49.5 without any step) and dearer for all others
+// (p_12 0.3115, p_24 13.58 -> 13.69, s_{8,8} 0.622 -> 0.631).  Returns the entries left.
+static __device__ __noinline__ unsigned axis_add(int m, int lcap, int64_t* buf, unsigned n, bool mine, int64_t at,
+                                                 double2* cand, unsigned flush) {
+  axis_push(buf, n, mine, at);
+  if (n >= flush) {
+    int64_t i;
+    if (axis_pop(buf, n, i)) cand[i] = axis_step(m, lcap, cand[i]);
+  }
+  return n;
+}
+
 // LIST: the starts list[0 .. *nlist) only (start list[t] for queue entry
 // t); the queue is ctr->queue_head2 then.  CAP: P has a captured term
 // (s_{l,n}).
 template <bool LIST, bool CAP>
 __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __restrict__ starts,
-                                                 int64_t count, float tol2, int cap,
+                                                 int64_t count, float tol2, int cap, unsigned axis_lo,
                                                  double2* __restrict__ cand,
                                                  uint8_t* __restrict__ status, DevCounters* ctr,
                                                  const uint32_t* __restrict__ list = nullptr,
@@ -42,10 +57,6 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
   __shared__ int64_t axis_buf[4][64];
   int64_t* abuf = axis_buf[threadIdx.x >> 5];
   unsigned na = 0;
-  auto axis = [&]() {
-    int64_t i;
-    if (axis_pop(abuf, na, i)) cand[i] = axis_step(P.m, P.lcap, cand[i]);
-  };
   for (;;) {
     // Lanes that finished are written and refilled together, once DESC_REFILL
     // of them wait or none is running: both cost a pass of the warp however
@@ -58,7 +69,7 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
       if (outcome >= 0) {
         const double2 z = descent_point(d);
         cand[at] = z;
-        near = outcome == 0 && d.fx && fx_below(z.y, AXIS_EXP);
+        near = outcome == 0 && d.fx && axis_near(z, axis_lo);
         status[at] = (uint8_t)outcome;
         nconv += outcome == 0;
         ndiv += outcome == 1;
@@ -66,8 +77,7 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
         outcome = -1;
         idx = -1;
       }
-      axis_push(abuf, na, near, at);
-      if (na >= 32u) axis();
+      if (__any_sync(0xffffffffu, near)) na = axis_add(P.m, P.lcap, abuf, na, near, at, cand, 32u);
       const unsigned need = drained ? 0u : __ballot_sync(0xffffffffu, idx < 0);
       if (need) {
         unsigned long long base = 0;
@@ -94,7 +104,7 @@ __global__ void __launch_bounds__(128) k_descend(PolyDev P, const double2* __res
       ++steps;
     }
   }
-  if (na) axis();
+  if (na) axis_add(P.m, P.lcap, abuf, na, false, 0, cand, 1u);
   warp_add_u64(&ctr->desc_newton, steps);
   if (!LIST) {  // a list's outcomes are counted where it joins the others
     warp_add_u64(&ctr->n_conv, nconv);
@@ -286,7 +296,7 @@ int device_sm_count() {
 }
 
 cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t count, double tol,
-                           int cap, double2* cand, uint8_t* status, DevCounters* ctr, int block,
+                           int cap, double eps, double2* cand, uint8_t* status, DevCounters* ctr, int block,
                            cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   const int bs = 128;
@@ -300,7 +310,8 @@ cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t coun
   // p_n, s_{l,n} (integer pipes): 24 warps per SM hide the multiply-adds'
   // latency; more only lengthen the tail in which a warp waits for its last
   // descents.  Measured: p_20 3 blocks 0.89 ms, 4 0.85, 5 0.84, 6 0.84, 8
-  // 0.87; p_24 15.6, 14.4, 13.9, 13.6, 13.4.
+  // 0.87; p_24 15.6, 14.4, 13.9, 13.6, 13.4 (at 8 1.5 % less there, 3 % more at
+  // p_20: one number for both).
   // q_{l,n} and the polynomials kept in binary64 (that pipe: 2 lanes per SM)
   // are saturated by 8 warps per SM (s_{2,16}: 0.72 ms, 1.13 with 24).
   const int most = P.kind == 2 || !P.fx ? 2 : 6;
@@ -313,13 +324,13 @@ cudaError_t launch_descend(const PolyDev& P, const double2* starts, int64_t coun
   if (P.kind == 2)
     k_descend_q<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol * tol, cap, cand, status, ctr);
   else
-    kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, cand, status, ctr, nullptr, nullptr);
+    kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, axis_floor(eps), cand, status, ctr, nullptr, nullptr);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return ktimer_end(s);
 }
 
 cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const uint32_t* list,
-                                const unsigned long long* nlist, int64_t count, double tol, int cap,
+                                const unsigned long long* nlist, int64_t count, double tol, int cap,double eps, 
                                 double2* cand, uint8_t* status, DevCounters* ctr, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   if (P.kind == 2) return cudaErrorInvalidValue;  // q_{l,n} has no mixed tier
@@ -336,7 +347,7 @@ cudaError_t launch_descend_list(const PolyDev& P, const double2* starts, const u
   if ((e = cudaMemsetAsync(&ctr->queue_head2, 0, sizeof(ctr->queue_head2), s)) != cudaSuccess) return e;
   MT_COUNT_LAUNCH(1);
   if ((e = ktimer_begin(KS_DESC64, s)) != cudaSuccess) return e;
-  kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, cand, status, ctr, list, nlist);
+  kd<<<(unsigned)grid, bs, 0, s>>>(P, starts, count, tol2_f(tol), cap, axis_floor(eps), cand, status, ctr, list, nlist);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return ktimer_end(s);
 }
