@@ -67,8 +67,9 @@ typedef enum {
 
 typedef enum {
   MT_FP64 = 0,   /* every step in 64 bits: fixed point, binary64 outside its range */
-  MT_MIXED = 1,  /* binary32 level-line tracking and early Newton, binary64 finish */
-  MT_DD = 2      /* binary64 with double-double for the clustered roots          */
+  MT_MIXED = 1,  /* binary32 level-line tracking and early Newton, 64-bit finish
+                    (p_23 to p_25: fixed point; else binary64)                    */
+  MT_DD = 2      /* the same with double-double for the clustered roots          */
 } mt_precision;
 
 /* Options.  Fill with mt_default_options() and override fields. */
@@ -149,7 +150,7 @@ typedef struct {
   int64_t desc_fp32;       /* binary32 Newton steps of the descents                */
   float ms_seeds;          /* device time of the seed lifts (part of ms_walk)      */
   int32_t reserved;
-  int64_t n_finish;        /* binary64 finishes in the mixed tier (one per run of
+  int64_t n_finish;        /* 64-bit finishes in the mixed tier (one per run of
                               descents that reached the same root in binary32)   */
   int64_t n_mult;          /* roots counted with multiplicity (q_{l,n}; n_roots
                               for the polynomials with simple roots)            */
@@ -158,10 +159,10 @@ typedef struct {
      launches; 0 where the kernel did not run or was not timed.  For the
      roofline of each kernel against the FMA rate of its own pipe. */
   float ms_k_walk;         /* the level-line walk (k_walk / k_walk_mixed)         */
-  float ms_k_desc64;       /* binary64 descents (k_descend; mixed tier: the tip redo) */
+  float ms_k_desc64;       /* 64-bit descents (k_descend; mixed tier: the tip redo) */
   float ms_k_desc32;       /* binary32 descents of the mixed tier (k_descend_mixed) */
-  float ms_k_finish;       /* binary64 finish of the mixed tier (k_finish_f64)    */
-  int64_t finish_newton;   /* binary64 Newton steps of k_finish_f64               */
+  float ms_k_finish;       /* 64-bit finish of the mixed tier (k_finish_f64)      */
+  int64_t finish_newton;   /* Newton steps of k_finish_f64                        */
   int32_t n_k_timed;       /* kernel launches timed in the four fields above      */
   int32_t n_tip64;         /* mixed tier: descents that ended within 1e-3 of the
                               left tip c = -2 and were redone in binary64 from
